@@ -9,6 +9,7 @@
 // graph: one block folds the per-file words into per-worker disagreement
 // masks in shared memory and writes adj = complement.
 #include "aspis_internal.cuh"
+#include "detect_common.cuh"
 
 namespace aspis {
 namespace {
@@ -116,20 +117,8 @@ graph_kernel(const uint32_t *__restrict__ file_neq, const uint8_t *__restrict__ 
     if (threadIdx.x < 32) dis[threadIdx.x] = 0;
     __syncthreads();
     for (int64_t i = threadIdx.x; i < f; i += blockDim.x) {
-        uint32_t w = file_neq[i];
-        while (w) {
-            int rem = __ffs(w) - 1;
-            w &= w - 1;
-            int s = 0;
-            while (rem >= r - 1 - s) {
-                rem -= r - 1 - s;
-                ++s;
-            }
-            const int t = s + 1 + rem;
-            const int a = fw[i * r + s], b = fw[i * r + t];
-            atomicOr(&dis[a], 1u << b);
-            atomicOr(&dis[b], 1u << a);
-        }
+        const uint32_t w = file_neq[i];
+        if (w) add_disagreements(w, fw + i * r, r, dis);
     }
     __syncthreads();
     if (threadIdx.x < (unsigned)K) {

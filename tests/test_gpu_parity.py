@@ -213,6 +213,21 @@ def test_detect_moon_moser(parts):
     assert got.clique_mask == sum(1 << (3 * p) for p in range(parts))
 
 
+@pytest.mark.parametrize("attack", ["weak", "strong"])
+def test_detect_attack_graphs(attack):
+    """Nearly complete graphs, which the search's closure step settles: every
+    (K, q) with 2 q <= K, r = 3."""
+    for K in range(3, 32):
+        for q in range(1, K // 2 + 1):
+            w = synth.Workload("g", K=K, r=3, d=1, q=q, attack=attack, seed=K + 40 * q)
+            adj = np.array(synth.attack_graph(w), np.uint32)
+            want = oracle.max_cliques_bk(adj, K)
+            got = detect_gpu(adj, K)
+            assert got.status == ap.OK, (K, q)
+            assert (got.omega, got.n_max_cliques, got.clique_mask) == \
+                (want.omega, want.n_max, want.clique), (K, q)
+
+
 def test_detect_degenerate_graphs():
     for K in (2, 3, 17, 31):
         got = detect_gpu(np.zeros(K, np.uint32), K)
