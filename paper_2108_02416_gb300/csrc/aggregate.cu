@@ -84,77 +84,6 @@ __device__ __forceinline__ typename Vec<V>::T load_row(const float *p)
     else return __ldcg(reinterpret_cast<const unsigned int *>(p));
 }
 
-// Histogram increment.  No memory clobber: the counters are read only after a
-// block barrier, so ordinary loads and stores may move across these.
-template <uint32_t INC>
-__device__ __forceinline__ void red_shared(uint32_t saddr)
-{
-    asm volatile("red.shared.add.u32 [%0], %1;\n" ::"r"(saddr), "n"(INC));
-}
-
-__device__ __forceinline__ void cp_async4(uint32_t saddr, const void *g)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(saddr), "l"(g) : "memory");
-}
-
-__device__ __forceinline__ void prefetch_l2(const void *p)
-{
-    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p));
-}
-
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// ascending bitonic sorting network over N registers (N a power of two)
-template <int N>
-__device__ __forceinline__ void sort_net(uint32_t (&y)[N])
-{
-#pragma unroll
-    for (int k = 2; k <= N; k <<= 1)
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1)
-#pragma unroll
-            for (int i = 0; i < N; ++i) {
-                const int l = i ^ j;
-                if (l > i) {
-                    const uint32_t a = y[i], b = y[l];
-                    const bool up = (i & k) == 0;
-                    y[i] = up ? min(a, b) : max(a, b);
-                    y[l] = up ? max(a, b) : min(a, b);
-                }
-            }
-}
-
-// the 32 values of a warp (one per lane) sorted ascending across the lanes
-// (bitonic: lane i meets lane i ^ j; the lower lane of an ascending block
-// keeps the minimum)
-__device__ __forceinline__ uint32_t warp_sort32(uint32_t x, int lane)
-{
-#pragma unroll
-    for (int k = 2; k <= 32; k <<= 1)
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
-            const bool up = (lane & k) == 0, lower = (lane & j) == 0;
-            x = lower == up ? min(x, y) : max(x, y);
-        }
-    return x;
-}
-
-// flag |= 1 if any of a, b, c, e is NaN (one compare per pair)
-__device__ __forceinline__ void nan_check(uint32_t &flag, float a, float b, float c, float e)
-{
-    asm("{\n .reg .pred p;\n setp.nan.f32 p, %1, %2;\n setp.nan.or.f32 p, %3, %4, p;\n"
-        " @p mov.b32 %0, 1;\n}\n" : "+r"(flag) : "f"(a), "f"(b), "f"(c), "f"(e));
-}
-
-// the low bytes of four words, packed into one word
-__device__ __forceinline__ uint32_t pack4(uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3)
-{
-    return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
-}
-
 template <int V>
 struct Geo {
     static constexpr int TC = 32 * V;                 // coordinates per tile
@@ -1036,14 +965,6 @@ median_radix_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t 
     }
 }
 
-size_t smem_cap()
-{
-    int dev = 0, cap = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return (size_t)cap - 1024;        // static shared memory and reserve
-}
-
 template <int V, int MINB, bool W32, int MODE, int NT>
 cudaError_t try_launch(bool &launched, const float *copies, int64_t f, int r, int64_t d,
                        int64_t ld, const int8_t *sel, aspis_detection *det, float *out,
@@ -1096,33 +1017,24 @@ cudaError_t launch_mode(int align, const float *copies, int64_t f, int r, int64_
     e = try_launch<V, MB, W32, MODE, NT>(ok, copies, f, r, d, ld, sel, det, out, stream);       \
     if (e != cudaSuccess || ok) return e;
     if (align >= 4) {
-        ASPIS_TRY(4, 2, 384)
-    }
-    if (align >= 2) {
-        ASPIS_TRY(2, 2, 384)
-    }
-    if (align >= 4) {
         ASPIS_TRY(4, 1, 384)
     }
     if (align >= 2) {
         ASPIS_TRY(2, 1, 384)
     }
-    if constexpr (MODE == 0) {
-        // more files than the tag bytes of 64-coordinate tiles hold: two
-        // passes over 128-coordinate tiles (twice the reads, 512-byte row
-        // segments) before the narrow one-pass tiles
-        if (align >= 4) {
-            e = try_launch<4, 2, W32, 2, 384>(ok, copies, f, r, d, ld, sel, det, out, stream);
-            if (e != cudaSuccess || ok) return e;
-            e = try_launch<4, 1, W32, 2, 384>(ok, copies, f, r, d, ld, sel, det, out, stream);
-            if (e != cudaSuccess || ok) return e;
-        }
+    // more files than the tag bytes of 64-coordinate tiles hold: two passes
+    // over 128-coordinate tiles (twice the reads, 512-byte row segments)
+    // before the narrow one-pass tiles
+    if (align >= 4) {
+        e = try_launch<4, 2, W32, 2, 384>(ok, copies, f, r, d, ld, sel, det, out, stream);
+        if (e != cudaSuccess || ok) return e;
+        e = try_launch<4, 1, W32, 2, 384>(ok, copies, f, r, d, ld, sel, det, out, stream);
+        if (e != cudaSuccess || ok) return e;
     }
     ASPIS_TRY(1, 2, 384)
     ASPIS_TRY(1, 1, 384)
 #undef ASPIS_TRY
-    if constexpr (MODE == 0) return launch_radix(copies, f, r, d, ld, sel, det, out, stream);
-    return cudaErrorInvalidValue;
+    return launch_radix(copies, f, r, d, ld, sel, det, out, stream);
 }
 
 }  // namespace
@@ -1132,15 +1044,16 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, i
                              cudaStream_t stream)
 {
     if (f > ASPIS_MAX_AGG_FILES || f * r > 65535) return cudaErrorInvalidValue;
+    // the tiles of round.cu for means and for medians of up to 640 files
+    bool done = false;
+    const cudaError_t e = launch_aggregate_tiles(done, copies, f, r, d, ld, sel, det, mode, out, stream, nullptr);
+    if (e != cudaSuccess || done) return e;
     // widest load every row start allows: 16 bytes (V = 4), 8 (V = 2), else 4
     const uintptr_t p = (uintptr_t)copies;
     const int align = (p % 16 == 0 && ld % 4 == 0) ? 4 : (p % 8 == 0 && ld % 2 == 0) ? 2 : 1;
     const bool w32 = (uint64_t)ld * 4u < (1ull << 32);     // row pitch fits a 32-bit multiplier
-    if (mode == 0)
-        return w32 ? launch_mode<0, true>(align, copies, f, r, d, ld, sel, det, out, stream)
-                   : launch_mode<0, false>(align, copies, f, r, d, ld, sel, det, out, stream);
-    return w32 ? launch_mode<1, true>(align, copies, f, r, d, ld, sel, det, out, stream)
-               : launch_mode<1, false>(align, copies, f, r, d, ld, sel, det, out, stream);
+    return w32 ? launch_mode<0, true>(align, copies, f, r, d, ld, sel, det, out, stream)
+               : launch_mode<0, false>(align, copies, f, r, d, ld, sel, det, out, stream);
 }
 
 }  // namespace aspis

@@ -25,6 +25,14 @@ int sm_count()
     return cached[dev];
 }
 
+size_t smem_cap()
+{
+    int dev = 0, cap = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return (size_t)cap - 1024;        // static shared memory and reserve
+}
+
 }  // namespace aspis
 
 using namespace aspis;
@@ -297,9 +305,16 @@ extern "C" aspis_status aspis_round(const float *copies, int64_t d, int64_t ld,
     if (!file_neq || !adj || !det || !sel || !out || (mode != 0 && mode != 1))
         return ASPIS_E_INVAL;
     if (a->f > ASPIS_MAX_AGG_FILES) return ASPIS_E_RANGE;
-    if ((s = aspis_check(copies, d, ld, a, file_neq, adj, stream)) != ASPIS_OK) return s;
-    if ((s = aspis_detect(adj, a->K, det, stream)) != ASPIS_OK) return s;
-    if ((s = aspis_select(file_neq, det, a, sel, stream)) != ASPIS_OK) return s;
+    bool done = false;
+    s = cuda_status(launch_round_fused(done, copies, a->f, a->r, a->K, d, ld, a->dev_file_workers,
+                                       file_neq, adj, det, sel, mode, out, (cudaStream_t)stream));
+    if (s != ASPIS_OK || done) return s;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (cudaMemsetAsync(file_neq, 0, sizeof(uint32_t) * (size_t)a->f, st) != cudaSuccess)
+        return ASPIS_E_CUDA;
+    if ((s = cuda_status(launch_compare(copies, a->f, a->r, d, ld, file_neq, st))) != ASPIS_OK) return s;
+    s = cuda_status(launch_decide(file_neq, a->dev_file_workers, a->f, a->r, a->K, adj, det, sel, st));
+    if (s != ASPIS_OK) return s;
     return aspis_aggregate(copies, d, ld, a, sel, det, mode, out, stream);
 }
 

@@ -21,9 +21,27 @@ cudaError_t launch_select(const uint32_t *file_neq, aspis_detection *det,
 cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d,
                              int64_t ld, const int8_t *sel, aspis_detection *det,
                              int mode, float *out, cudaStream_t stream);
+// Step 5 in 128-coordinate tiles (round.cu); done = false where the median's
+// tag bytes of f files do not fit a block.  gate: see round.cu, or NULL.
+cudaError_t launch_aggregate_tiles(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
+                                   const int8_t *sel, aspis_detection *det, int mode, float *out,
+                                   cudaStream_t stream, aspis_detection *gate);
+// Steps 2-4 (graph, maximum cliques, selection) in one launch, for f <=
+// ASPIS_MAX_AGG_FILES.
+cudaError_t launch_decide(uint32_t *file_neq, const uint8_t *dev_file_workers, int64_t f, int r, int K,
+                          uint32_t *adj, aspis_detection *det, int8_t *sel, cudaStream_t stream);
+// The whole round in one pass over the copies; done = false (and nothing
+// enqueued) where the separate steps have to run.
+cudaError_t launch_round_fused(bool &done, const float *copies, int64_t f, int r, int K, int64_t d,
+                               int64_t ld, const uint8_t *dev_file_workers, uint32_t *file_neq,
+                               uint32_t *adj, aspis_detection *det, int8_t *sel, int mode,
+                               float *out, cudaStream_t stream);
 
 // Number of SMs of the current device (cached per device).
 int sm_count();
+
+// Dynamic shared memory a block may ask for on the current device.
+size_t smem_cap();
 
 __host__ __device__ inline int pair_count(int r) { return r * (r - 1) / 2; }
 

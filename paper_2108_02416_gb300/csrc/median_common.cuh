@@ -38,7 +38,7 @@ __device__ __forceinline__ uint32_t vbin_bits(float x, float s, float c)
     return __float_as_uint(fmaf(y, (float)kTopBin, 8388608.0f));
 }
 
-enum { M_DONE = 0, M_VH, M_VC, M_VM, M_KA, M_KH, M_KC };
+enum { M_DONE = 0, M_VH, M_VC, M_VM, M_KV, M_KA, M_KH, M_KC };
 
 // Four tag bytes against the target bytes of vbx: 0x80 in each byte whose tag
 // equals its target, 0 elsewhere.  Exact for every byte value: the sum of a
@@ -57,6 +57,77 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
     s = a + b;
     const float bp = s - a;
     e = (a - (s - bp)) + (b - bp);
+}
+
+// Histogram increment.  No memory clobber: the counters are read only after a
+// block barrier, so ordinary loads and stores may move across these.
+template <uint32_t INC>
+__device__ __forceinline__ void red_shared(uint32_t saddr)
+{
+    asm volatile("red.shared.add.u32 [%0], %1;\n" ::"r"(saddr), "n"(INC));
+}
+
+__device__ __forceinline__ void cp_async4(uint32_t saddr, const void *g)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(saddr), "l"(g) : "memory");
+}
+
+__device__ __forceinline__ void prefetch_l2(const void *p)
+{
+    asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p));
+}
+
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+// ascending bitonic sorting network over N registers (N a power of two)
+template <int N>
+__device__ __forceinline__ void sort_net(uint32_t (&y)[N])
+{
+#pragma unroll
+    for (int k = 2; k <= N; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1)
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const int l = i ^ j;
+                if (l > i) {
+                    const uint32_t a = y[i], b = y[l];
+                    const bool up = (i & k) == 0;
+                    y[i] = up ? min(a, b) : max(a, b);
+                    y[l] = up ? max(a, b) : min(a, b);
+                }
+            }
+}
+
+// the 32 values of a warp (one per lane) sorted ascending across the lanes
+// (bitonic: lane i meets lane i ^ j; the lower lane of an ascending block
+// keeps the minimum)
+__device__ __forceinline__ uint32_t warp_sort32(uint32_t x, int lane)
+{
+#pragma unroll
+    for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
+            const bool up = (lane & k) == 0, lower = (lane & j) == 0;
+            x = lower == up ? min(x, y) : max(x, y);
+        }
+    return x;
+}
+
+// flag |= 1 if any of a, b, c, e is NaN (one compare per pair)
+__device__ __forceinline__ void nan_check(uint32_t &flag, float a, float b, float c, float e)
+{
+    asm("{\n .reg .pred p;\n setp.nan.f32 p, %1, %2;\n setp.nan.or.f32 p, %3, %4, p;\n"
+        " @p mov.b32 %0, 1;\n}\n" : "+r"(flag) : "f"(a), "f"(b), "f"(c), "f"(e));
+}
+
+// the low bytes of four words, packed into one word
+__device__ __forceinline__ uint32_t pack4(uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3)
+{
+    return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
 }
 
 }  // namespace aspis

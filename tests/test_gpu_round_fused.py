@@ -1,0 +1,124 @@
+"""The round in one pass over the copies (taken from 100 million values of
+copies on): every step's output against the CPU oracle on the same bytes, for
+selections that the sampled coordinates show, for distortions that they miss
+(the aggregate is then made again), for ragged and unaligned rows, and for
+values that need the median's exact passes."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+from _gpu_round import assert_mean_close, assert_round_matches, gpu_round
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+ap = pytest.importorskip("paper_2108_02416_gb300")
+DEV = torch.device("cuda:0")
+VALUES = 100_000_000
+
+
+def build(K, r, d, q, attack, seed, ld=None):
+    """Host copies [f, r, ld]: normal gradients, the adversaries' copies shifted."""
+    oa = oracle.assign(K, r)
+    rng = np.random.default_rng(seed)
+    ld = d if ld is None else ld
+    host = np.empty((oa.f, r, ld), np.float32)
+    g = rng.standard_normal((oa.f, ld), dtype=np.float32)
+    host[:] = g[:, None, :]
+    w = synth.Workload("x", K=K, r=r, d=d, q=q, attack=attack, seed=seed)
+    mask = synth.corrupted_mask(w, oa.file_workers)
+    return oa, host, mask
+
+
+def check(oa, host, d, mode=0, offset=0):
+    want = oracle.run_round(host, oa, d, mode)
+    a = ap.aspis_assign(oa.K, oa.r)
+    flat = torch.empty(host.size + offset, dtype=torch.float32, device=DEV)
+    dev = flat[offset:].view(host.shape)
+    dev.copy_(torch.from_numpy(host))
+    buf = gpu_round(ap, torch, dev, d, a, mode)
+    assert_round_matches(ap, buf, want, mode, check_out=mode == 0)
+    if mode == 1:
+        rows = np.array([host[i, s, :d] for i, s in enumerate(want.sel) if s >= 0])
+        assert_mean_close(buf.out.cpu().numpy(), want.out, np.abs(rows.astype(np.float64)).mean(0))
+    return buf
+
+
+def smallest_d(K, r):
+    return -(-VALUES // (oracle.assign(K, r).f * r))
+
+
+CLUSTERS = [(7, 3, 2), (15, 2, 5), (15, 3, 3), (10, 4, 4), (12, 4, 5), (10, 5, 3)]
+
+
+@pytest.mark.parametrize("K,r,q", CLUSTERS)
+@pytest.mark.parametrize("attack,mode", [("strong", 0), ("weak", 0), ("weak", 1)])
+def test_seen_distortions(K, r, q, attack, mode):
+    d = smallest_d(K, r) + 1
+    oa, host, mask = build(K, r, d, q, attack, 10 * K + r, ld=(d + 3) // 4 * 4)
+    host[mask] = -3.0 * host[mask]
+    check(oa, host, d, mode)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("attack", ["strong", "weak"])
+@pytest.mark.parametrize("K,r,q", [(15, 3, 3), (10, 5, 3)])
+def test_distortions_outside_the_sample(K, r, q, attack, mode):
+    """Each corrupted copy differs at one coordinate only, and the values of
+    slot 0 lie far from the others' there."""
+    d = smallest_d(K, r) + 2
+    oa, host, mask = build(K, r, d, q, attack, K + r, ld=(d + 3) // 4 * 4)
+    rng = np.random.default_rng(1)
+    for i, s in zip(*np.nonzero(mask)):
+        host[i, s, int(rng.choice([0, 1, d - 1, int(rng.integers(d))]))] += np.float32(100.0)
+    check(oa, host, d, mode)
+
+
+@pytest.mark.parametrize("extra,offset", [(0, 0), (1, 0), (2, 0), (31, 0), (64, 1), (127, 3)])
+def test_rows_at_any_address(extra, offset):
+    d = smallest_d(15, 3) // 128 * 128 + 128 + extra
+    oa, host, mask = build(15, 3, d, 3, "strong", extra + 5)
+    host[mask] += np.float32(0.5)
+    check(oa, host, d, offset=offset)
+
+
+def test_padding_and_exact_passes():
+    """Padding that differs between copies, and coordinates of equal values,
+    two values, NaNs, infinities, signed zeros and subnormals."""
+    K, r = 15, 3
+    d = smallest_d(K, r) + 1
+    ld = (d + 3) // 4 * 4 + 4
+    oa, host, mask = build(K, r, d, 3, "weak", 3, ld=ld)
+    f = oa.f
+    rng = np.random.default_rng(2)
+    u = host.view(np.uint32)
+    u[:, :, 5] = 0x3F800000
+    u[:, :, 6] = np.where(np.arange(f) % 2, 0x3F800000, 0xBF800000)[:, None]
+    u[:, :, 700] = np.where(np.arange(f) % 3, 0x00000000, 0x80000000)[:, None]
+    u[:, :, 701] = (np.arange(f) % 7)[:, None]
+    u[3, :, 900] = 0x7FC00001
+    u[4, :, 1000] = 0xFFC00000
+    u[::2, :, 1100] = 0x7F800000
+    u[1::2, :, 1101] = 0xFF800000
+    host[:, :, d - 1] = 1.0 + 1e-6 * np.arange(f)[:, None] * (np.arange(f)[:, None] % 50 == 0)
+    host[mask] += np.float32(1e-3)
+    host[:, :, d:] = rng.standard_normal((f, r, ld - d))
+    buf = check(oa, host, d)
+    assert buf.detection().median_exact > 0
+
+
+def test_guess_of_an_earlier_round_is_not_kept():
+    """Two rounds on the same buffers, the second with other adversaries."""
+    d = smallest_d(15, 3)
+    a = ap.aspis_assign(15, 3)
+    buf = ap.RoundBuffers(a, d, DEV)
+    for seed in (1, 2):
+        oa, host, mask = build(15, 3, d, 3, "weak", seed)
+        host[mask] += np.float32(1.0)
+        want = oracle.run_round(host, oa, d, 0)
+        ap.aspis_round(torch.from_numpy(host).to(DEV), d, a, buf.file_neq, buf.adj, buf.det, buf.sel, buf.out)
+        torch.cuda.synchronize()
+        assert_round_matches(ap, buf, want)
