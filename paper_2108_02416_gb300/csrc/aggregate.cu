@@ -1,5 +1,6 @@
-// Step 5 of the PS round: coordinate-wise aggregation of the chosen copies
-// (Algorithm 1: median of the majority gradients; mean in Case 1).
+// Step 5 of the PS round for more files than the tiles of sweep_impl.cuh hold
+// tags for (kTagFiles): the coordinate-wise lower median of the chosen copies
+// in narrower tiles or in two passes.
 //
 // Data path.  A tile is TC = 32*V consecutive coordinates (V = 4, 2 or 1) of
 // all n kept rows.  Lane l of every warp holds coordinates [l*V, l*V + V) of
@@ -110,7 +111,7 @@ __host__ __device__ inline Layout make_layout(int64_t f)
     const int64_t per_slot = (f + kWarps - 1) / kWarps;
     const int64_t jw = (per_slot + G::RPW - 1) / G::RPW;     // tag words per thread
     size_t o = 0;
-    // the mean and the two-pass median keep no tags
+    // the two-pass median keeps no tags
     L.tags = o; o += MODE == 0 ? (size_t)jw * kWarps * 32 * 4 : 0;
     L.hist = o; o += (size_t)G::HW * 4;
     L.list = o; o += (size_t)(MODE == 2 ? kListWords2 : kListWords) * 4;   // also the partial sums
@@ -357,39 +358,7 @@ aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, 
             batch(std::true_type{}, j0);
         };
 
-        if constexpr (MODE == 1) {
-            // ---- mean: compensated per-thread sums, combined in warp order
-            float sm[V], se[V];
-#pragma unroll
-            for (int k = 0; k < V; ++k) sm[k] = se[k] = 0.f;
-            sweep([](int) {}, [&](const T &x, int, int) {
-#pragma unroll
-                for (int k = 0; k < V; ++k) {
-                    float ns, ne;
-                    two_sum(sm[k], __uint_as_float(elem<V>(x, k)), ns, ne);
-                    sm[k] = ns;
-                    se[k] += ne;
-                }
-            }, std::false_type{});
-#pragma unroll
-            for (int k = 0; k < V; ++k) {
-                list[(2 * w) * TC + lane * V + k] = __float_as_uint(sm[k]);
-                list[(2 * w + 1) * TC + lane * V + k] = __float_as_uint(se[k]);
-            }
-            __syncthreads();
-            for (int c = tid; c < TC; c += kThreads) {
-                if (c0 + c >= d) continue;
-                float a = 0.f, ae = 0.f;
-                for (int u = 0; u < kWarps; ++u) {
-                    float ns, ne;
-                    two_sum(a, __uint_as_float(list[(2 * u) * TC + c]), ns, ne);
-                    a = ns;
-                    ae += ne + __uint_as_float(list[(2 * u + 1) * TC + c]);
-                }
-                out[c0 + c] = (float)(((double)a + (double)ae) / (double)n);
-            }
-            __syncthreads();
-        } else {
+        {
             // ---- S: key range of the sample (rows 0 and 1 of every warp)
             if (lv) {
 #pragma unroll
@@ -827,7 +796,7 @@ aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, 
             }
         }
     }
-    if constexpr (MODE != 1) {
+    {
         // the last tile's listed members are ranked once their copies land
         if (MODE == 0 && have_p) {
             cp_async_wait_all();
@@ -1007,53 +976,42 @@ cudaError_t launch_radix(const float *copies, int64_t f, int r, int64_t d, int64
     return cudaGetLastError();
 }
 
-template <int MODE, bool W32>
-cudaError_t launch_mode(int align, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
+template <bool W32>
+cudaError_t launch_many(int align, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
                         const int8_t *sel, aspis_detection *det, float *out, cudaStream_t stream)
 {
     bool ok = false;
     cudaError_t e = cudaSuccess;
-#define ASPIS_TRY(V, MB, NT)                                                                    \
-    e = try_launch<V, MB, W32, MODE, NT>(ok, copies, f, r, d, ld, sel, det, out, stream);       \
+#define ASPIS_TRY(V, MB, MODE)                                                                  \
+    e = try_launch<V, MB, W32, MODE, 384>(ok, copies, f, r, d, ld, sel, det, out, stream);      \
     if (e != cudaSuccess || ok) return e;
-    if (align >= 4) {
-        ASPIS_TRY(4, 1, 384)
-    }
     if (align >= 2) {
-        ASPIS_TRY(2, 1, 384)
+        ASPIS_TRY(2, 1, 0)
     }
     // more files than the tag bytes of 64-coordinate tiles hold: two passes
     // over 128-coordinate tiles (twice the reads, 512-byte row segments)
     // before the narrow one-pass tiles
     if (align >= 4) {
-        e = try_launch<4, 2, W32, 2, 384>(ok, copies, f, r, d, ld, sel, det, out, stream);
-        if (e != cudaSuccess || ok) return e;
-        e = try_launch<4, 1, W32, 2, 384>(ok, copies, f, r, d, ld, sel, det, out, stream);
-        if (e != cudaSuccess || ok) return e;
+        ASPIS_TRY(4, 2, 2)
+        ASPIS_TRY(4, 1, 2)
     }
-    ASPIS_TRY(1, 2, 384)
-    ASPIS_TRY(1, 1, 384)
+    ASPIS_TRY(1, 2, 0)
+    ASPIS_TRY(1, 1, 0)
 #undef ASPIS_TRY
     return launch_radix(copies, f, r, d, ld, sel, det, out, stream);
 }
 
 }  // namespace
 
-cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, int64_t ld,
-                             const int8_t *sel, aspis_detection *det, int mode, float *out,
-                             cudaStream_t stream)
+cudaError_t launch_aggregate_many(const float *copies, int64_t f, int r, int64_t d, int64_t ld,
+                                  const int8_t *sel, aspis_detection *det, float *out, cudaStream_t stream)
 {
-    if (f > ASPIS_MAX_AGG_FILES || f * r > 65535) return cudaErrorInvalidValue;
-    // the tiles of round.cu for means and for medians of up to 640 files
-    bool done = false;
-    const cudaError_t e = launch_aggregate_tiles(done, copies, f, r, d, ld, sel, det, mode, out, stream, nullptr);
-    if (e != cudaSuccess || done) return e;
     // widest load every row start allows: 16 bytes (V = 4), 8 (V = 2), else 4
     const uintptr_t p = (uintptr_t)copies;
     const int align = (p % 16 == 0 && ld % 4 == 0) ? 4 : (p % 8 == 0 && ld % 2 == 0) ? 2 : 1;
     const bool w32 = (uint64_t)ld * 4u < (1ull << 32);     // row pitch fits a 32-bit multiplier
-    return w32 ? launch_mode<0, true>(align, copies, f, r, d, ld, sel, det, out, stream)
-               : launch_mode<0, false>(align, copies, f, r, d, ld, sel, det, out, stream);
+    return w32 ? launch_many<true>(align, copies, f, r, d, ld, sel, det, out, stream)
+               : launch_many<false>(align, copies, f, r, d, ld, sel, det, out, stream);
 }
 
 }  // namespace aspis

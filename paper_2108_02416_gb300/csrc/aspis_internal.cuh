@@ -18,14 +18,14 @@ cudaError_t launch_detect(const uint32_t *adj, int K, aspis_detection *det,
 cudaError_t launch_select(const uint32_t *file_neq, aspis_detection *det,
                           const uint8_t *dev_file_workers, int64_t f, int r,
                           int8_t *sel, cudaStream_t stream);
+// gate: a repair of the one-pass round (round.cu), or NULL.
 cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d,
                              int64_t ld, const int8_t *sel, aspis_detection *det,
-                             int mode, float *out, cudaStream_t stream);
-// Step 5 in 128-coordinate tiles (round.cu); done = false where the median's
-// tag bytes of f files do not fit a block.  gate: see round.cu, or NULL.
-cudaError_t launch_aggregate_tiles(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
-                                   const int8_t *sel, aspis_detection *det, int mode, float *out,
-                                   cudaStream_t stream, aspis_detection *gate);
+                             int mode, float *out, cudaStream_t stream,
+                             aspis_detection *gate = nullptr);
+// The lower median for f > kTagFiles (aggregate.cu).
+cudaError_t launch_aggregate_many(const float *copies, int64_t f, int r, int64_t d, int64_t ld,
+                                  const int8_t *sel, aspis_detection *det, float *out, cudaStream_t stream);
 // Steps 2-4 (graph, maximum cliques, selection) in one launch, for f <=
 // ASPIS_MAX_AGG_FILES.
 cudaError_t launch_decide(uint32_t *file_neq, const uint8_t *dev_file_workers, int64_t f, int r, int K,

@@ -38,7 +38,7 @@ __device__ __forceinline__ uint32_t vbin_bits(float x, float s, float c)
     return __float_as_uint(fmaf(y, (float)kTopBin, 8388608.0f));
 }
 
-enum { M_DONE = 0, M_VH, M_VC, M_VM, M_KV, M_KA, M_KH, M_KC };
+enum { M_DONE = 0, M_VH, M_VC, M_VM, M_KA, M_KH, M_KC };
 
 // Four tag bytes against the target bytes of vbx: 0x80 in each byte whose tag
 // equals its target, 0 elsewhere.  Exact for every byte value: the sum of a

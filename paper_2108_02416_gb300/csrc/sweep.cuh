@@ -1,0 +1,54 @@
+// One pass over the copies in tiles of 128 coordinates: all pairs of copies
+// compared, the chosen copies aggregated (R > 1: R copies per file, in the
+// file's rows; R = 1: one row per file, only aggregated).
+//
+// Lower median, exact (IEEE totalOrder through a monotone uint32 key; the key
+// map is a bijection, so the output has the chosen element's bits).  Lane l of
+// every warp holds four coordinates of the tile, the warps split the files.
+//   sample  24 values per coordinate give the span of 255 value bins
+//   sweep   every value's bin is counted (8-bit counters, four coordinates per
+//           word, 32 banks) and kept as a tag byte
+//   search  the bin that holds the median's rank
+//   list    the bin's members (about n / 100), found by their tags, copied
+//           into the coordinate's list while the next tile is swept
+//   rank    the lists are ranked after it
+// What this cannot settle (a NaN, an overflowed counter, a crowded bin, no
+// spread in the sample) is left open for fixup_kernel.
+//
+// More than kTagFiles files leave no room for tags: the sweep then only counts,
+// and a second pass over the chosen rows lists the members.  (Sharing a tile
+// among the blocks of a cluster, counters and members exchanged through
+// distributed shared memory, kept one pass but cost 15 to 25 us per tile: 6.9
+// against 6.2 ms at 3,003 files of five copies and d = 2^19.)
+#pragma once
+
+#include <utility>
+
+#include "aspis_internal.cuh"
+#include "median_common.cuh"
+
+namespace aspis {
+
+constexpr int64_t kTagFiles = 1330;         // most files whose tag bytes leave a tile room in a block
+constexpr int kUnclean = 16;                // in a guessed sel: copies of the file differ
+// Bits of a coordinate that the sweep leaves to fixup_kernel.  They may also
+// be a median's own bits (a NaN payload): computing that one again gives it.
+constexpr uint32_t kOpen = 0x7FA5C3E1u;
+
+struct SweepArgs {
+    const float *copies;
+    int64_t d, ld;
+    int f;
+    const int8_t *sel;
+    aspis_detection *det;
+    float *out;
+    uint32_t *file_neq;              // R > 1: pair words, ORed
+    int r;                           // R = 1: row i * r + sel[i] is file i's
+    aspis_detection *gate;           // R = 1: run only where a repair was asked for, or NULL
+};
+
+// ok = false where no layout holds f files (median, more than about 6,000).
+template <int R>
+cudaError_t launch_sweep(bool &ok, const SweepArgs &A, int mode, bool vec, cudaStream_t stream);
+
+}  // namespace aspis

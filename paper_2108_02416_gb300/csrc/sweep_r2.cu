@@ -1,0 +1,6 @@
+// sweep_kernel for 2 copies per file.
+#include "sweep_impl.cuh"
+
+namespace aspis {
+template cudaError_t launch_sweep<2>(bool &, const SweepArgs &, int, bool, cudaStream_t);
+}  // namespace aspis

@@ -110,6 +110,17 @@ def test_padding_and_exact_passes():
     assert buf.detection().median_exact > 0
 
 
+@pytest.mark.parametrize("K,r,q,pad", [(21, 3, 4, 0), (24, 3, 5, 1), (15, 5, 4, 3)])
+def test_many_files(K, r, q, pad):
+    """One block per SM (1,330 files), and two passes without tags beyond that
+    (taken from a thousand million values on); ragged rows, aligned or not."""
+    f = oracle.assign(K, r).f
+    d = -(-(VALUES if f <= 1330 else 10 * VALUES) // (f * r)) | 1
+    oa, host, mask = build(K, r, d, q, "strong", K, ld=d + pad)
+    host[mask] *= np.float32(-10.0)
+    check(oa, host, d)
+
+
 def test_guess_of_an_earlier_round_is_not_kept():
     """Two rounds on the same buffers, the second with other adversaries."""
     d = smallest_d(15, 3)
