@@ -23,6 +23,12 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d,
                              int64_t ld, const int8_t *sel, aspis_detection *det,
                              int mode, float *out, cudaStream_t stream,
                              aspis_detection *gate = nullptr);
+// Averages of the copies in slot_mask into means (16-byte aligned rows) and
+// their lower median in one pass; done = false (and nothing enqueued) where the
+// separate passes are better or the only ones.
+cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
+                                  const uint8_t *slot_mask, const int8_t *sel, float *means, int64_t ldm,
+                                  aspis_detection *det, float *out, cudaStream_t stream);
 // The lower median for f > kTagFiles (aggregate.cu).
 cudaError_t launch_aggregate_many(const float *copies, int64_t f, int r, int64_t d, int64_t ld,
                                   const int8_t *sel, aspis_detection *det, float *out, cudaStream_t stream);

@@ -130,4 +130,33 @@ __device__ __forceinline__ uint32_t pack4(uint32_t b0, uint32_t b1, uint32_t b2,
     return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
 }
 
+// mean of the values x[s] of the slots s in m (fp32: x0 plus the
+// mean of the deviations from it; 0 where a copy equals x0 bit for bit); s0 = the
+// lowest slot of m, k = |m|; every index is a compile-time slot
+template <int R>
+__device__ __forceinline__ float mean_masked(const float (&x)[R], uint32_t m, int s0, int k)
+{
+    if (k == R) {                          // all copies: nothing to pick, a constant divisor
+        const uint32_t b = __float_as_uint(x[0]);
+        float sum = 0.f;
+#pragma unroll
+        for (int s = 1; s < R; ++s)
+            sum = __fadd_rn(sum, __float_as_uint(x[s]) == b ? 0.f : __fsub_rn(x[s], x[0]));
+        return sum == 0.f ? x[0] : __fadd_rn(x[0], __fdiv_rn(sum, (float)R));
+    }
+    float x0 = x[0];
+#pragma unroll
+    for (int s = 1; s < R; ++s)
+        if (s == s0) x0 = x[s];
+    const uint32_t b0 = __float_as_uint(x0);
+    float acc = 0.f;
+#pragma unroll
+    for (int s = 0; s < R; ++s)
+        if ((m >> s) & 1u) {
+            const float e = __float_as_uint(x[s]) == b0 ? 0.f : __fsub_rn(x[s], x0);
+            acc = __fadd_rn(acc, e);
+        }
+    return acc == 0.f ? x0 : __fadd_rn(x0, __fdiv_rn(acc, (float)k));
+}
+
 }  // namespace aspis

@@ -72,6 +72,7 @@ sample_kernel(const uint32_t *__restrict__ copies, int64_t f, int64_t d, int64_t
 
 constexpr int kDecideThreads = 1024;
 constexpr int64_t kMinValues = 100'000'000;  // fp32 values of the smallest round taken in one pass
+constexpr int64_t kMinAverages = 20'000'000; // and of the smallest averages that feed the median directly
 
 // Steps 2-4 in one block (f <= ASPIS_MAX_AGG_FILES): three launches less than
 // the separate kernels, which take 3 + 4..18 + 3 us one after the other.
@@ -353,7 +354,7 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, i
 {
     if (f > ASPIS_MAX_AGG_FILES || f * r > 65535) return cudaErrorInvalidValue;
     const bool vec = (uintptr_t)copies % 16 == 0 && ld % 4 == 0;
-    const SweepArgs A{copies, d, ld, (int)f, sel, det, out, nullptr, r, gate};
+    const SweepArgs A{copies, d, ld, (int)f, sel, det, out, nullptr, r, gate, nullptr, nullptr, 0};
     // Many files: one pass over narrow tiles (92 us, and 28 more for the open
     // coordinates, against 28 at 2,024 files, d = 9,000) or two passes with
     // more rows in flight (165 against 126 us at 3,003 files).
@@ -363,6 +364,28 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, i
     if (e != cudaSuccess) return e;
     if (!ok) return cudaErrorInvalidValue;
     return mode == 0 ? launch_fixup(A, stream) : cudaSuccess;
+}
+
+cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
+                                  const uint8_t *slot_mask, const int8_t *sel, float *means, int64_t ldm,
+                                  aspis_detection *det, float *out, cudaStream_t stream)
+{
+    done = false;
+    // (62 against 54 us at 455 files of three and d = 4,096, 73 against 75 at
+    // 16,384, 176 against 199 at 65,536)
+    if (r > 5 || f > kTagFiles || f * r * d < kMinAverages) return cudaSuccess;
+    const SweepArgs A{copies, d, ld, (int)f, sel, det, out, nullptr, r, nullptr, slot_mask, means, ldm};
+    cudaError_t e;
+    switch (r) {
+    case 2: e = launch_sweep_averages<2>(done, A, stream); break;
+    case 3: e = launch_sweep_averages<3>(done, A, stream); break;
+    case 4: e = launch_sweep_averages<4>(done, A, stream); break;
+    default: e = launch_sweep_averages<5>(done, A, stream); break;
+    }
+    if (e != cudaSuccess || !done) return e;
+    // open coordinates: from the averages, one row per file
+    const SweepArgs F{means, d, ldm, (int)f, sel, det, out, nullptr, 1, nullptr, nullptr, nullptr, 0};
+    return launch_fixup(F, stream);
 }
 
 cudaError_t launch_decide(uint32_t *file_neq, const uint8_t *fw, int64_t f, int r, int K, uint32_t *adj,
@@ -396,7 +419,7 @@ cudaError_t launch_round_fused(bool &done, const float *copies, int64_t f, int r
     // 881 for the separate steps at 2,024 files of three, d = 131,072; 6.56
     // against 5.64 ms at d = 2^20.
     if (mode == 0 && f > kTagFiles && f * r * d < 10 * kMinValues) return cudaSuccess;
-    const SweepArgs A{copies, d, ld, (int)f, sel, det, out, file_neq, r, nullptr};
+    const SweepArgs A{copies, d, ld, (int)f, sel, det, out, file_neq, r, nullptr, nullptr, nullptr, 0};
     switch (r) {
     case 2: return fused<2>(done, A, fw, K, adj, sel, mode, vec, stream);
     case 3: return fused<3>(done, A, fw, K, adj, sel, mode, vec, stream);

@@ -45,10 +45,18 @@ struct SweepArgs {
     uint32_t *file_neq;              // R > 1: pair words, ORed
     int r;                           // R = 1: row i * r + sel[i] is file i's
     aspis_detection *gate;           // R = 1: run only where a repair was asked for, or NULL
+    const uint8_t *slot_mask;        // averages: the copies averaged per file,
+    float *means;                    // and where their averages go, [f][ldm]
+    int64_t ldm;
 };
 
 // ok = false where no layout holds f files (median, more than about 6,000).
 template <int R>
 cudaError_t launch_sweep(bool &ok, const SweepArgs &A, int mode, bool vec, cudaStream_t stream);
+
+// The median of the averages of the copies in slot_mask, which are also written
+// to means (R > 1, aligned rows, f <= kTagFiles); nothing is compared.
+template <int R>
+cudaError_t launch_sweep_averages(bool &ok, const SweepArgs &A, cudaStream_t stream);
 
 }  // namespace aspis

@@ -176,7 +176,9 @@ __device__ __forceinline__ int warp_ranked(uint32_t a, uint32_t b, uint32_t cnt,
     return 0;
 }
 
-template <int R, bool VEC, int MODE, int MINB>
+// AVG: a file's value is the average of its copies in slot_mask; the meta word
+// holds the mask in place of slot and pair word.
+template <int R, bool VEC, int MODE, int MINB, bool AVG = false>
 __global__ void __launch_bounds__(kNT, MINB)
 sweep_kernel(const SweepArgs A)
 {
@@ -262,7 +264,10 @@ sweep_kernel(const SweepArgs A)
         }
     } else {
         if constexpr (MODE != MEAN) {
-            for (int i = tid; i < f; i += kNT) list[i] = A.sel[i] < 0 || A.sel[i] >= kUnclean ? 0x80000000u : 0u;
+            for (int i = tid; i < f; i += kNT) {
+                const bool marked = AVG ? A.slot_mask[i] != (1u << R) - 1u : A.sel[i] < 0 || A.sel[i] >= kUnclean;
+                list[i] = marked ? 0x80000000u : 0u;
+            }
             __syncthreads();
             start = cleanest_start(list, f, &start_s);
         }
@@ -270,8 +275,9 @@ sweep_kernel(const SweepArgs A)
         for (int i = tid; i < f; i += kNT) {
             const int s = A.sel[i];
             meta[(i < start ? f : 0) + i - start] =
-                (uint32_t)(s < 0 ? kDropped : s & (kUnclean - 1)) | ((uint32_t)i << 16);
-            mine += s >= 0;
+                (AVG ? (uint32_t)A.slot_mask[i] : (uint32_t)(s < 0 ? kDropped : s & (kUnclean - 1))) |
+                ((uint32_t)i << 16);
+            mine += AVG ? A.slot_mask[i] != 0 : s >= 0;
         }
         mine = __reduce_add_sync(full, mine);
         if (lane == 0 && mine) atomicAdd(&n_s, mine);
@@ -288,7 +294,11 @@ sweep_kernel(const SweepArgs A)
     const int nf = R == 1 ? n : f;                                    // files of a tile
     const int nmine = nf > w ? (nf - w + kWarps - 1) / kWarps : 0;    // of this warp
     auto word_of = [&](int j) -> uint32_t { return meta[w + j * kWarps]; };
-    auto slot_of = [&](int j) -> int { return R == 1 ? 0 : (int)(word_of(j) & 15u); };
+    // the slot of the chosen (AVG: of the first averaged) copy
+    auto slot_of = [&](int j) -> int {
+        if constexpr (AVG) return word_of(j) & 0xFFu ? __ffs((int)(word_of(j) & 0xFFu)) - 1 : kDropped;
+        return R == 1 ? 0 : (int)(word_of(j) & 15u);
+    };
     // a file's copies start here, from the lane's base in row 0
     auto file_at = [&](const char *base, int j) -> const char * {
         return base + (uint64_t)(R == 1 ? word_of(j) : (word_of(j) >> 16) * R) * ldb;
@@ -316,9 +326,10 @@ sweep_kernel(const SweepArgs A)
             if (kl > 3) x.w = __ldcg(e + 96);
         }
     };
-    auto load_file = [&](uint4 (&x)[R], const char *p, int kl) {
+    auto load_file = [&](uint4 (&x)[R], const char *p, int kl, uint32_t mask) {
 #pragma unroll
         for (int s = 0; s < R; ++s) {
+            if (AVG && !((mask >> s) & 1u)) continue;
             const char *q = p + (uint64_t)s * ldb;
             if constexpr (VEC) {
                 // the copies of slot 0 are the usual choice: they stay in L2
@@ -339,7 +350,7 @@ sweep_kernel(const SweepArgs A)
         for (int u = 0; u < kF; ++u) {
 #pragma unroll
             for (int s = 0; s < R; ++s) xa[u][s] = make_uint4(0u, 0u, 0u, 0u);
-            if (u < nmine) load_file(xa[u], file_at(p, u), kl);
+            if (u < nmine) load_file(xa[u], file_at(p, u), kl, word_of(u));
         }
     }
 
@@ -417,7 +428,7 @@ sweep_kernel(const SweepArgs A)
 #pragma unroll
             for (int q0 = 0; q0 < kRows * 4; q0 += 32) {
                 const int q = q0 + lane, row = q / 4, jp = j + row / R;
-                if (q < kRows * 4 && jp < nmine && cb + (q & 3) * 32 < d)
+                if (q < kRows * 4 && jp < nmine && cb + (q & 3) * 32 < d && (!AVG || (word_of(jp) >> (row % R)) & 1u))
                     prefetch_l2(file_at(reinterpret_cast<const char *>(A.copies + cb + (q & 3) * 32), jp) +
                                 (uint64_t)(row % R) * ldb);
             }
@@ -435,6 +446,32 @@ sweep_kernel(const SweepArgs A)
             auto file = [&](uint4 (&x)[R], int j) {
                 if constexpr (R == 1) {
                     fn(x[0], j);
+                    return;
+                }
+                if constexpr (AVG) {
+                    const uint32_t m = word_of(j) & 0xFFu;
+                    if (!m) {
+                        skip(j);
+                        return;
+                    }
+                    const int s0 = __ffs((int)m) - 1, many = __popc(m);
+                    uint32_t v[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        float a[R];
+#pragma unroll
+                        for (int s = 0; s < R; ++s) a[s] = __uint_as_float(el(x[s], k));
+                        v[k] = __float_as_uint(mean_masked<R>(a, m, s0, many));
+                    }
+                    float *to = A.means + (int64_t)(word_of(j) >> 16) * A.ldm + c0 + lane * 4;
+                    if (kl == 4) {
+                        __stcg(reinterpret_cast<uint4 *>(to), make_uint4(v[0], v[1], v[2], v[3]));
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 3; ++k)
+                            if (k < kl) to[k] = __uint_as_float(v[k]);
+                    }
+                    fn(make_uint4(v[0], v[1], v[2], v[3]), j);
                     return;
                 }
                 if (ragged) mask_tail(x);
@@ -466,7 +503,7 @@ sweep_kernel(const SweepArgs A)
                 for (int u = 0; u < kF; ++u) {
                     file(xa[u], j0 + u);
                     const int jn = j0 + kF + u;
-                    if (jn < nmine) load_file(xa[u], file_at(lb, jn), kl);
+                    if (jn < nmine) load_file(xa[u], file_at(lb, jn), kl, word_of(jn));
                 }
             }
 #pragma unroll
@@ -476,7 +513,7 @@ sweep_kernel(const SweepArgs A)
 #pragma unroll
                     for (int s = 0; s < R; ++s) load_chosen(xa[u][s], u * R + s);
                 } else {
-                    if (u < nmine) load_file(xa[u], file_at(lbn, u), kln);
+                    if (u < nmine) load_file(xa[u], file_at(lbn, u), kln, word_of(u));
                 }
             }
         };
@@ -717,7 +754,7 @@ sweep_kernel(const SweepArgs A)
                 for (int u = 0; u < kF; ++u) {
 #pragma unroll
                     for (int s = 0; s < R; ++s) take(xa[u][s], j0 + u * R + s);
-                    if (u < nmine) load_file(xa[u], file_at(lbn, u), kln);
+                    if (u < nmine) load_file(xa[u], file_at(lbn, u), kln, word_of(u));
                 }
                 if (tn < ntiles) prefetch_batch(tn * TC, kF);
                 __syncthreads();
@@ -742,7 +779,9 @@ sweep_kernel(const SweepArgs A)
                         const uint32_t at = atomicAdd(&S(S_LCNT, c), 1u);
                         if (at < (uint32_t)kCap)
                             cp_async4(list_s + (at * TC + c) * 4u,
-                                      file_at(lb, j) + (uint64_t)slot_of(j) * ldb + (VEC ? k : 32 * k) * 4);
+                                      AVG ? reinterpret_cast<const char *>(A.means + (int64_t)(word_of(j) >> 16) * A.ldm +
+                                                                           c0 + c)
+                                          : file_at(lb, j) + (uint64_t)slot_of(j) * ldb + (VEC ? k : 32 * k) * 4);
                     }
                 }
                 cp_async_commit();
@@ -768,7 +807,7 @@ sweep_kernel(const SweepArgs A)
     }
     if constexpr (R == 1) {
         if (tid == 0) gate_leave(A.gate);
-    } else {
+    } else if constexpr (!AVG) {
         for (int i = tid; i < f; i += kNT) {
             const uint32_t neq = (meta[i] >> 4) & 0xFFFu;
             if (neq) atomicOr(&A.file_neq[meta[i] >> 16], neq);
@@ -776,13 +815,13 @@ sweep_kernel(const SweepArgs A)
     }
 }
 
-template <int R, bool VEC, int MODE, int MINB>
+template <int R, bool VEC, int MODE, int MINB, bool AVG = false>
 cudaError_t try_sweep(bool &ok, const SweepArgs &A, cudaStream_t stream)
 {
     ok = false;
     const SweepLayout L = sweep_layout<MODE>(A.f);
     if (L.total > smem_cap()) return cudaSuccess;
-    auto kern = sweep_kernel<R, VEC, MODE, MINB>;
+    auto kern = sweep_kernel<R, VEC, MODE, MINB, AVG>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -821,6 +860,16 @@ template <int R>
 cudaError_t launch_sweep(bool &ok, const SweepArgs &A, int mode, bool vec, cudaStream_t stream)
 {
     return vec ? sweep_for<R, true>(ok, A, mode, stream) : sweep_for<R, false>(ok, A, mode, stream);
+}
+
+template <int R>
+cudaError_t launch_sweep_averages(bool &ok, const SweepArgs &A, cudaStream_t stream)
+{
+    ok = false;
+    cudaError_t e = cudaSuccess;
+    if ((A.d + TC - 1) / TC > sm_count()) e = try_sweep<R, true, TAGGED, 2, true>(ok, A, stream);
+    if (e == cudaSuccess && !ok) e = try_sweep<R, true, TAGGED, 1, true>(ok, A, stream);
+    return e;
 }
 
 }  // namespace aspis

@@ -22,6 +22,7 @@
 // close slot pairs, at most 28 bits), file_mean (streams the chosen copies
 // of every kept file once and writes one row per file).
 #include "aspis_internal.cuh"
+#include "median_common.cuh"
 
 namespace {
 
@@ -186,26 +187,6 @@ select_tol_kernel(const uint32_t *__restrict__ file_neq, aspis_detection *det,
     if (threadIdx.x == 0 && kept) atomicAdd(&det->n_sel, kept);
 }
 
-// mean of the values x[s] of the slots s in m (reading above); s0 = the
-// lowest slot of m, k = |m|; every index is a compile-time slot
-template <int R>
-__device__ __forceinline__ float mean_masked(const float (&x)[R], uint32_t m, int s0, int k)
-{
-    float x0 = x[0];
-#pragma unroll
-    for (int s = 1; s < R; ++s)
-        if (s == s0) x0 = x[s];
-    const uint32_t b0 = __float_as_uint(x0);
-    float acc = 0.f;
-#pragma unroll
-    for (int s = 0; s < R; ++s)
-        if ((m >> s) & 1u) {
-            const float e = __float_as_uint(x[s]) == b0 ? 0.f : __fsub_rn(x[s], x0);
-            acc = __fadd_rn(acc, e);
-        }
-    return acc == 0.f ? x0 : __fadd_rn(x0, __fdiv_rn(acc, (float)k));
-}
-
 // Grid-stride over (file, chunk of kThreads * 4 float4 or floats); only the
 // chosen copies of a kept file are read, once, and their mean is written to
 // means[i * ldm + c].
@@ -306,6 +287,16 @@ cudaError_t launch_tolerant(const float *copies, int64_t f, int64_t d, int64_t l
         file_neq, det, fw, f, slot_mask, sel);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const bool vmean = vec && (uintptr_t)means % 16 == 0 && ldm % 4 == 0;
+    // averages and median in one pass over the chosen copies: the median takes
+    // the averages from the registers that they are written from (2.41 -> 2.12
+    // ms for the round at 455 files of three and d = 2^20; the mean gained
+    // nothing, 2.31 against 2.28: tiles of 512-byte segments write less
+    // efficiently than whole rows)
+    if (vmean && mode == 0) {
+        bool done = false;
+        e = launch_average_median(done, copies, f, R, d, ld, slot_mask, sel, means, ldm, det, out, st);
+        if (e != cudaSuccess || done) return e;
+    }
     if (vmean) {
         const int64_t per = (int64_t)kThreads * 4 * 4;
         const int64_t nch = (d + per - 1) / per;

@@ -124,6 +124,33 @@ def test_tolerant_unaligned_paths(offset, ldm_pad):
     check(run(host, w, 1e-4, 0, offset, ldm_pad), want, host, 0)
 
 
+@pytest.mark.parametrize("K,r,q,attack", [(15, 2, 4, "weak"), (15, 3, 4, "strong"), (15, 3, 4, "weak"),
+                                          (10, 4, 4, "weak"), (10, 5, 4, "strong"), (21, 3, 4, "weak")])
+@pytest.mark.parametrize("extra", [1, 64])
+def test_averages_feed_the_median(K, r, q, attack, extra):
+    """From 20 million copies' values on the averages go straight into the
+    median: subsets of the slots averaged, files dropped (their rows of means
+    left as they were), coordinates of equal values and a NaN, ragged tails."""
+    f = oracle.assign(K, r).f
+    d = 20_000_000 // (f * r) // 128 * 128 + 128 + extra
+    w = synth.Workload("avg", K=K, r=r, d=d, q=q, attack=attack, seed=K + r)
+    oa = oracle.assign(K, r)
+    rng = np.random.default_rng(r)
+    host = np.zeros((f, r, (d + 3) // 4 * 4), np.float32)
+    host[:] = rng.standard_normal((f, 1, host.shape[2]), dtype=np.float32)
+    host += 1e-6 * rng.standard_normal(host.shape, dtype=np.float32)
+    host[:, :, 7] = 2.5
+    mask = synth.corrupted_mask(w, oa.file_workers)
+    host[mask] = -10.0 * host[mask]
+    # (a NaN and no infinity: the comparison below subtracts, and infinities
+    # that agree would not pass it)
+    host[2, :, 300] = np.float32(np.nan)
+    want = oracle.run_round_tolerant(host, oa, 1e-4, d, 0)
+    buf = run(host, w, 1e-4)
+    check(buf, want, host)
+    assert not buf.means[torch.from_numpy(want.slot_mask == 0).to(DEV)].any()
+
+
 @pytest.mark.parametrize("K,r,q,attack", [(6, 2, 2, "weak"), (8, 2, 3, "strong"), (8, 4, 3, "strong"),
                                           (9, 4, 4, "weak"), (9, 6, 4, "strong")])
 def test_tolerant_other_r(K, r, q, attack):
