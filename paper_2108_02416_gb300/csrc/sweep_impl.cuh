@@ -315,15 +315,16 @@ sweep_kernel(const SweepArgs A)
         const int64_t q = VEC ? left - lane * 4 : (left - lane + 31) / 32;
         return q < 0 ? 0 : q > 4 ? 4 : (int)q;
     };
+    // (the four 128-byte pieces of an unaligned row share lines: through L1)
     auto load_row = [&](uint4 &x, const char *p, int kl) {
         if constexpr (VEC) {
             if (kl > 0) x = __ldcg(reinterpret_cast<const uint4 *>(p));
         } else {
             const unsigned int *e = reinterpret_cast<const unsigned int *>(p);
-            if (kl > 0) x.x = __ldcg(e);
-            if (kl > 1) x.y = __ldcg(e + 32);
-            if (kl > 2) x.z = __ldcg(e + 64);
-            if (kl > 3) x.w = __ldcg(e + 96);
+            if (kl > 0) x.x = __ldca(e);
+            if (kl > 1) x.y = __ldca(e + 32);
+            if (kl > 2) x.z = __ldca(e + 64);
+            if (kl > 3) x.w = __ldca(e + 96);
         }
     };
     auto load_file = [&](uint4 (&x)[R], const char *p, int kl, uint32_t mask) {
@@ -331,13 +332,18 @@ sweep_kernel(const SweepArgs A)
         for (int s = 0; s < R; ++s) {
             if (AVG && !((mask >> s) & 1u)) continue;
             const char *q = p + (uint64_t)s * ldb;
-            if constexpr (VEC) {
-                // the copies of slot 0 are the usual choice: they stay in L2
-                // for the member lists, the others are first to go
-                const uint4 *e = reinterpret_cast<const uint4 *>(q);
-                if (kl > 0) x[s] = s == 0 ? __ldcg(e) : __ldcs(e);
-            } else {
+            // the copies of slot 0 are the usual choice: they stay in L2 for
+            // the member lists, the others are first to go
+            if (s == 0 || (!VEC && MODE == MEAN)) {
                 load_row(x[s], q, kl);
+            } else if constexpr (VEC) {
+                if (kl > 0) x[s] = __ldcs(reinterpret_cast<const uint4 *>(q));
+            } else {
+                const unsigned int *e = reinterpret_cast<const unsigned int *>(q);
+                if (kl > 0) x[s].x = __ldcs(e);
+                if (kl > 1) x[s].y = __ldcs(e + 32);
+                if (kl > 2) x[s].z = __ldcs(e + 64);
+                if (kl > 3) x[s].w = __ldcs(e + 96);
             }
         }
     };
@@ -423,13 +429,17 @@ sweep_kernel(const SweepArgs A)
                 if (kl < 4) x[s].w = 0u;
             }
         };
-        // files j.. of a batch into L2, one 128-byte line per lane
+        // files j.. of a batch into L2, one 128-byte line per lane.  An
+        // unaligned segment lies in five lines; the fifth is left to the next
+        // tile where it would take one more instruction per batch (which cost
+        // 3 to 5% with two or four copies; without it three copies lost 14%).
+        constexpr int kLines = !VEC && MODE != MEAN && (kRows * 5 + 31) / 32 == (kRows * 4 + 31) / 32 ? 5 : 4;
         auto prefetch_batch = [&](int64_t cb, int j) {
 #pragma unroll
-            for (int q0 = 0; q0 < kRows * 4; q0 += 32) {
-                const int q = q0 + lane, row = q / 4, jp = j + row / R;
-                if (q < kRows * 4 && jp < nmine && cb + (q & 3) * 32 < d && (!AVG || (word_of(jp) >> (row % R)) & 1u))
-                    prefetch_l2(file_at(reinterpret_cast<const char *>(A.copies + cb + (q & 3) * 32), jp) +
+            for (int q0 = 0; q0 < kRows * kLines; q0 += 32) {
+                const int q = q0 + lane, row = q / kLines, col = q % kLines * 32, jp = j + row / R;
+                if (q < kRows * kLines && jp < nmine && cb + col < d && (!AVG || (word_of(jp) >> (row % R)) & 1u))
+                    prefetch_l2(file_at(reinterpret_cast<const char *>(A.copies + cb + col), jp) +
                                 (uint64_t)(row % R) * ldb);
             }
         };
