@@ -321,7 +321,7 @@ cudaError_t launch_fixup(const SweepArgs &A, cudaStream_t stream)
 
 template <int R>
 cudaError_t fused(bool &done, const SweepArgs &A, const uint8_t *fw, int K, uint32_t *adj, int8_t *sel,
-                  int mode, bool vec, cudaStream_t stream)
+                  int mode, cudaStream_t stream)
 {
     sample_kernel<R><<<(unsigned)((A.f + 3) / 4), kSampleThreads, 0, stream>>>(
         reinterpret_cast<const uint32_t *>(A.copies), A.f, A.d, A.ld, A.file_neq);
@@ -330,7 +330,7 @@ cudaError_t fused(bool &done, const SweepArgs &A, const uint8_t *fw, int K, uint
     decide_kernel<R, GUESS><<<1, kDecideThreads, 0, stream>>>(A.file_neq, fw, A.f, K, adj, A.det, sel);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     bool ok = false;
-    if ((e = launch_sweep<R>(ok, A, mode, vec, stream)) != cudaSuccess) return e;
+    if ((e = launch_sweep<R>(ok, A, mode, stream)) != cudaSuccess) return e;
     if (!ok) return cudaErrorInvalidValue;
     decide_kernel<R, VERIFY><<<1, kDecideThreads, 0, stream>>>(A.file_neq, fw, A.f, K, adj, A.det, sel);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -353,14 +353,13 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, i
                              aspis_detection *gate)
 {
     if (f > ASPIS_MAX_AGG_FILES || f * r > 65535) return cudaErrorInvalidValue;
-    const bool vec = (uintptr_t)copies % 16 == 0 && ld % 4 == 0;
     const SweepArgs A{copies, d, ld, (int)f, sel, det, out, nullptr, r, gate, nullptr, nullptr, 0};
     // Many files: one pass over narrow tiles (92 us, and 28 more for the open
     // coordinates, against 28 at 2,024 files, d = 9,000) or two passes with
     // more rows in flight (165 against 126 us at 3,003 files).
     if (mode == 0 && f > kTagFiles && !gate) return launch_aggregate_many(copies, f, r, d, ld, sel, det, out, stream);
     bool ok = false;
-    const cudaError_t e = launch_sweep<1>(ok, A, mode, vec, stream);
+    const cudaError_t e = launch_sweep<1>(ok, A, mode, stream);
     if (e != cudaSuccess) return e;
     if (!ok) return cudaErrorInvalidValue;
     return mode == 0 ? launch_fixup(A, stream) : cudaSuccess;
@@ -388,6 +387,29 @@ cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, in
     return launch_fixup(F, stream);
 }
 
+// Whether the one-pass round beats the separate compare and aggregation, from
+// the bytes that each moves and the rates measured for them (TB/s on GB300:
+// compare 7.1, sweep 6.3, the separate median 4.4, mean 5.6, median of more
+// than kTagFiles files 2.7) and the launches (the guess, its check and the
+// empty repair: 30 us against 10).  Tiles of 128 coordinates run one per
+// resident block at a time, and a last wave that is nearly empty costs about
+// 0.4 of a full one (its blocks have the bandwidth for themselves): the one-pass
+// mean of 3,003 files of five copies takes 550 us against 482 with 316 tiles
+// on 304 blocks, 1,309 against 1,355 with 1,024.
+bool one_pass_pays(int64_t f, int r, int64_t d, int mode)
+{
+    const bool many = mode == 0 && f > kTagFiles;                       // two passes over the chosen rows
+    if (f * r * d < (many ? 10 : 1) * kMinValues) return false;
+    const int64_t tiles = (d + 127) / 128;
+    const int64_t blocks = (int64_t)sm_count() * (mode == 1 || many || f <= kPairFiles ? 2 : 1);
+    const double full = (double)((tiles + blocks - 1) / blocks * blocks) / (double)tiles;
+    const double wave = 1.0 + 0.4 * (full - 1.0);
+    const double all = (double)f * r * (double)d * 4e-6, chosen = all / r;      // MB: us at 1 TB/s
+    const double once = (many ? all + chosen : all) / 6.3 * wave + 30.0;
+    const double apart = all / 7.1 + (many ? chosen / 2.7 : chosen / (mode == 1 ? 5.6 : 4.4) * wave) + 10.0;
+    return once < apart;
+}
+
 cudaError_t launch_decide(uint32_t *file_neq, const uint8_t *fw, int64_t f, int r, int K, uint32_t *adj,
                           aspis_detection *det, int8_t *sel, cudaStream_t stream)
 {
@@ -408,23 +430,13 @@ cudaError_t launch_round_fused(bool &done, const float *copies, int64_t f, int r
                                int8_t *sel, int mode, float *out, cudaStream_t stream)
 {
     done = false;
-    const bool vec = (uintptr_t)copies % 16 == 0 && ld % 4 == 0;
-    // The guess, its check and the empty repair cost about 20 us; the bytes
-    // not read again are worth that from about 350 MB of copies on (455 files
-    // of three: 102 us against 99 for the separate steps at 358 MB, 137
-    // against 142 at 537 MB).
-    if (r > 5 || f * r * d < kMinValues) return cudaSuccess;
-    // Beyond what tag bytes allow the median takes a second pass over the
-    // chosen rows even here, and only the first one is shared: 872 us against
-    // 881 for the separate steps at 2,024 files of three, d = 131,072; 6.56
-    // against 5.64 ms at d = 2^20.
-    if (mode == 0 && f > kTagFiles && f * r * d < 10 * kMinValues) return cudaSuccess;
+    if (r > 5 || !one_pass_pays(f, r, d, mode)) return cudaSuccess;
     const SweepArgs A{copies, d, ld, (int)f, sel, det, out, file_neq, r, nullptr, nullptr, nullptr, 0};
     switch (r) {
-    case 2: return fused<2>(done, A, fw, K, adj, sel, mode, vec, stream);
-    case 3: return fused<3>(done, A, fw, K, adj, sel, mode, vec, stream);
-    case 4: return fused<4>(done, A, fw, K, adj, sel, mode, vec, stream);
-    default: return fused<5>(done, A, fw, K, adj, sel, mode, vec, stream);
+    case 2: return fused<2>(done, A, fw, K, adj, sel, mode, stream);
+    case 3: return fused<3>(done, A, fw, K, adj, sel, mode, stream);
+    case 4: return fused<4>(done, A, fw, K, adj, sel, mode, stream);
+    default: return fused<5>(done, A, fw, K, adj, sel, mode, stream);
     }
 }
 

@@ -29,6 +29,7 @@
 
 namespace aspis {
 
+constexpr int64_t kPairFiles = 516;         // most files whose tag bytes let two blocks share an SM
 constexpr int64_t kTagFiles = 1330;         // most files whose tag bytes leave a tile room in a block
 constexpr int kUnclean = 16;                // in a guessed sel: copies of the file differ
 // Bits of a coordinate that the sweep leaves to fixup_kernel.  They may also
@@ -52,7 +53,7 @@ struct SweepArgs {
 
 // ok = false where no layout holds f files (median, more than about 6,000).
 template <int R>
-cudaError_t launch_sweep(bool &ok, const SweepArgs &A, int mode, bool vec, cudaStream_t stream);
+cudaError_t launch_sweep(bool &ok, const SweepArgs &A, int mode, cudaStream_t stream);
 
 // The median of the averages of the copies in slot_mask, which are also written
 // to means (R > 1, aligned rows, f <= kTagFiles); nothing is compared.

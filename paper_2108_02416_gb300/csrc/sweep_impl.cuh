@@ -27,8 +27,12 @@ constexpr int TC = 128;                     // coordinates per tile, four per la
 // What the sweep computes: the median with tag bytes, the mean, or the median
 // without tags, from a second pass over the chosen rows.
 enum Mode { TAGGED = 0, MEAN = 1, TWO_PASS = 2 };
-// list entries per coordinate
-__host__ __device__ constexpr int list_cap(int mode) { return mode == TWO_PASS ? 96 : 32; }
+// List entries per coordinate (CAP; the two-pass median's bins are wider).  A
+// bin has n / 120 members on average; half the list lets two blocks share the
+// SM up to kPairFiles files (456 with 32 entries), and 16 are hardly ever
+// exceeded there.
+template <int MODE, int CAP>
+__host__ __device__ constexpr int list_cap() { return MODE == TWO_PASS ? 96 : CAP; }
 constexpr int kHistWords = kVB * 32;        // four 8-bit counters per (bin, lane)
 constexpr int kBPW = (kVB + kWarps - 1) / kWarps;
 constexpr int kSample = 2 * kWarps;         // sampled values per coordinate
@@ -47,7 +51,7 @@ struct SweepLayout {
     size_t tags, hist, list, state, meta, total;
 };
 
-template <int MODE>
+template <int MODE, int CAP>
 __host__ __device__ inline SweepLayout sweep_layout(int64_t f)
 {
     SweepLayout L{};
@@ -56,18 +60,57 @@ __host__ __device__ inline SweepLayout sweep_layout(int64_t f)
     size_t o = 0;
     L.tags = o; o += MODE == TAGGED ? (size_t)per_warp * kWarps * 128 : 0;
     L.hist = o; o += MODE != MEAN ? (size_t)kHistWords * 4 : 0;
-    L.list = o; o += (size_t)list_cap(MODE) * TC * 4;      // (the mean: its partial sums)
+    L.list = o; o += (size_t)list_cap<MODE, CAP>() * TC * 4;      // (the mean: its partial sums)
     L.state = o; o += MODE != MEAN ? (size_t)kStateWords * TC * 4 : 0;
     L.meta = o; o += ((size_t)f * 4 + 15) / 16 * 16;
     L.total = o;
     return L;
 }
 
-// coordinate c of a tile (lane c / 4, element c % 4) in the tile's row segment
-template <bool VEC>
+// A row start is aligned to W floats (4, 2 or 1), the widest load it allows: a
+// lane holds W neighbouring coordinates of each of the 4 / W parts of the
+// tile's 128-float row segment.  off_of: element k of a lane, from its first;
+// seg_at: coordinate c of a tile (lane c / 4, element c % 4), from the tile's.
+template <int W>
+__host__ __device__ constexpr int off_of(int k)
+{
+    return k % W + k / W * 32 * W;
+}
+
+template <int W>
 __device__ __forceinline__ int seg_at(int c)
 {
-    return VEC ? c : (c >> 2) + 32 * (c & 3);
+    return (c >> 2) * W + off_of<W>(c & 3);
+}
+
+// the first kl elements of a lane (a pair or four are loaded whole: what lies
+// beyond d is padding of the same row)
+template <int W, bool STREAM>
+__device__ __forceinline__ void load_lane(uint4 &x, const char *p, int kl)
+{
+    if constexpr (W == 4) {
+        const uint4 *e = reinterpret_cast<const uint4 *>(p);
+        if (kl > 0) x = STREAM ? __ldcs(e) : __ldcg(e);
+    } else if constexpr (W == 2) {
+        const uint2 *e = reinterpret_cast<const uint2 *>(p);
+        if (kl > 0) {
+            const uint2 y = STREAM ? __ldcs(e) : __ldca(e);
+            x.x = y.x;
+            x.y = y.y;
+        }
+        if (kl > 2) {
+            const uint2 y = STREAM ? __ldcs(e + 32) : __ldca(e + 32);
+            x.z = y.x;
+            x.w = y.y;
+        }
+    } else {
+        // (the four 128-byte parts of an unaligned segment share lines: through L1)
+        const unsigned int *e = reinterpret_cast<const unsigned int *>(p);
+        if (kl > 0) x.x = STREAM ? __ldcs(e) : __ldca(e);
+        if (kl > 1) x.y = STREAM ? __ldcs(e + 32) : __ldca(e + 32);
+        if (kl > 2) x.z = STREAM ? __ldcs(e + 64) : __ldca(e + 64);
+        if (kl > 3) x.w = STREAM ? __ldcs(e + 96) : __ldca(e + 96);
+    }
 }
 
 __device__ __forceinline__ uint32_t el(const uint4 &x, int k)
@@ -178,24 +221,24 @@ __device__ __forceinline__ int warp_ranked(uint32_t a, uint32_t b, uint32_t cnt,
 
 // AVG: a file's value is the average of its copies in slot_mask; the meta word
 // holds the mask in place of slot and pair word.
-template <int R, bool VEC, int MODE, int MINB, bool AVG = false>
+template <int R, int W, int MODE, int MINB, bool AVG, int CAP>
 __global__ void __launch_bounds__(kNT, MINB)
 sweep_kernel(const SweepArgs A)
 {
     if (R == 1 && !gate_open(A.gate)) return;
-    constexpr int kCap = list_cap(MODE);
     constexpr int kShort = MINB == 1 || (MODE == TWO_PASS && R == 1) ? 16 : 8;   // longest list one thread sorts
     constexpr int kF = batch_files(R, MINB);
     constexpr int kRows = kF * R;
     static_assert(kF >= 2, "the sample is the first two files of every warp");
     extern __shared__ __align__(16) unsigned char smem[];
-    const SweepLayout L = sweep_layout<MODE>(A.f);
+    constexpr uint32_t cap = (uint32_t)list_cap<MODE, CAP>();
+    const SweepLayout L = sweep_layout<MODE, CAP>(A.f);
     uint32_t *tags = reinterpret_cast<uint32_t *>(smem + L.tags);     // [warp's file][kWarps][32]
     // the sampled keys: a warp's own first tag rows, which nothing else reads,
     // or (no tags) the list, empty at a tile's start
     uint32_t *keys = reinterpret_cast<uint32_t *>(smem + (MODE == TWO_PASS ? L.list : L.tags));
     uint32_t *hist = reinterpret_cast<uint32_t *>(smem + L.hist);     // [kVB][32]
-    uint32_t *list = reinterpret_cast<uint32_t *>(smem + L.list);     // [kCap][TC]
+    uint32_t *list = reinterpret_cast<uint32_t *>(smem + L.list);     // [cap][TC]
     uint32_t *st = reinterpret_cast<uint32_t *>(smem + L.state);      // [kStateWords][TC]
     // by place in the tile's order: slot | pair word << 4 | file << 16, or
     // (R = 1) the kept row
@@ -306,26 +349,16 @@ sweep_kernel(const SweepArgs A)
     // the lane's part of tile t: address in row 0, and how many of its four
     // coordinates exist
     auto lane_base = [&](int64_t t) -> const char * {
-        return reinterpret_cast<const char *>(A.copies + t * TC + (VEC ? lane * 4 : lane));
+        return reinterpret_cast<const char *>(A.copies + t * TC + lane * W);
     };
     auto live_of = [&](int64_t t) -> int {
         if (t >= ntiles) return 0;
         const int64_t left = d - t * TC;
         if (left >= TC) return 4;
-        const int64_t q = VEC ? left - lane * 4 : (left - lane + 31) / 32;
-        return q < 0 ? 0 : q > 4 ? 4 : (int)q;
-    };
-    // (the four 128-byte pieces of an unaligned row share lines: through L1)
-    auto load_row = [&](uint4 &x, const char *p, int kl) {
-        if constexpr (VEC) {
-            if (kl > 0) x = __ldcg(reinterpret_cast<const uint4 *>(p));
-        } else {
-            const unsigned int *e = reinterpret_cast<const unsigned int *>(p);
-            if (kl > 0) x.x = __ldca(e);
-            if (kl > 1) x.y = __ldca(e + 32);
-            if (kl > 2) x.z = __ldca(e + 64);
-            if (kl > 3) x.w = __ldca(e + 96);
-        }
+        int kl = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) kl += lane * W + off_of<W>(k) < left;
+        return kl;
     };
     auto load_file = [&](uint4 (&x)[R], const char *p, int kl, uint32_t mask) {
 #pragma unroll
@@ -334,17 +367,8 @@ sweep_kernel(const SweepArgs A)
             const char *q = p + (uint64_t)s * ldb;
             // the copies of slot 0 are the usual choice: they stay in L2 for
             // the member lists, the others are first to go
-            if (s == 0 || (!VEC && MODE == MEAN)) {
-                load_row(x[s], q, kl);
-            } else if constexpr (VEC) {
-                if (kl > 0) x[s] = __ldcs(reinterpret_cast<const uint4 *>(q));
-            } else {
-                const unsigned int *e = reinterpret_cast<const unsigned int *>(q);
-                if (kl > 0) x[s].x = __ldcs(e);
-                if (kl > 1) x[s].y = __ldcs(e + 32);
-                if (kl > 2) x[s].z = __ldcs(e + 64);
-                if (kl > 3) x[s].w = __ldcs(e + 96);
-            }
+            if (s == 0 || (W < 4 && MODE == MEAN)) load_lane<W, false>(x[s], q, kl);
+            else load_lane<W, true>(x[s], q, kl);
         }
     };
 
@@ -380,7 +404,7 @@ sweep_kernel(const SweepArgs A)
                 uint32_t res = y[0];
 #pragma unroll
                 for (int e = 1; e < kShort; ++e) res = (uint32_t)e == rk ? y[e] : res;
-                A.out[c0_p + seg_at<VEC>(c)] = __uint_as_float(from_key(res));
+                A.out[c0_p + seg_at<W>(c)] = __uint_as_float(from_key(res));
             }
         }
         const int nl = n_long[parity];
@@ -390,14 +414,14 @@ sweep_kernel(const SweepArgs A)
             if (MODE == TAGGED || cnt <= 32u) {
                 const uint32_t x = warp_sort32((uint32_t)lane < cnt ? to_key(list[lane * TC + c]) : 0xffffffffu, lane);
                 const uint32_t res = __shfl_sync(full, x, (int)rk);
-                if (lane == 0) A.out[c0_p + seg_at<VEC>(c)] = __uint_as_float(from_key(res));
+                if (lane == 0) A.out[c0_p + seg_at<W>(c)] = __uint_as_float(from_key(res));
                 continue;
             }
             if (cnt <= 64u) {
                 // (equal keys: several lanes write the same bits)
                 const uint32_t a = list[lane * TC + c], b = (uint32_t)lane + 32u < cnt ? list[(lane + 32) * TC + c] : 0u;
                 const int is = warp_ranked(to_key(a), to_key(b), cnt, rk);
-                if (is) A.out[c0_p + seg_at<VEC>(c)] = __uint_as_float(is == 1 ? a : b);
+                if (is) A.out[c0_p + seg_at<W>(c)] = __uint_as_float(is == 1 ? a : b);
                 continue;
             }
             for (uint32_t e = (uint32_t)lane; e < cnt; e += 32u) {
@@ -408,7 +432,7 @@ sweep_kernel(const SweepArgs A)
                     lt += y < x;
                     le += y <= x;
                 }
-                if (lt <= rk && rk < le) A.out[c0_p + seg_at<VEC>(c)] = __uint_as_float(from_key(x));
+                if (lt <= rk && rk < le) A.out[c0_p + seg_at<W>(c)] = __uint_as_float(from_key(x));
             }
         }
     };
@@ -433,7 +457,7 @@ sweep_kernel(const SweepArgs A)
         // unaligned segment lies in five lines; the fifth is left to the next
         // tile where it would take one more instruction per batch (which cost
         // 3 to 5% with two or four copies; without it three copies lost 14%).
-        constexpr int kLines = !VEC && MODE != MEAN && (kRows * 5 + 31) / 32 == (kRows * 4 + 31) / 32 ? 5 : 4;
+        constexpr int kLines = W < 4 && MODE != MEAN && (kRows * 5 + 31) / 32 == (kRows * 4 + 31) / 32 ? 5 : 4;
         auto prefetch_batch = [&](int64_t cb, int j) {
 #pragma unroll
             for (int q0 = 0; q0 < kRows * kLines; q0 += 32) {
@@ -450,7 +474,7 @@ sweep_kernel(const SweepArgs A)
         // second pass's first rows instead.)
         auto chosen_at = [&](int j) -> const char * { return file_at(lb, j) + (uint64_t)slot_of(j) * ldb; };
         auto load_chosen = [&](uint4 &x, int j) {
-            if (j < nmine && slot_of(j) != kDropped) load_row(x, chosen_at(j), kl);
+            if (j < nmine && slot_of(j) != kDropped) load_lane<W, false>(x, chosen_at(j), kl);
         };
         auto sweep = [&](auto fn, auto skip) {
             auto file = [&](uint4 (&x)[R], int j) {
@@ -548,7 +572,7 @@ sweep_kernel(const SweepArgs A)
                 list[(2 * w + 1) * TC + lane * 4 + k] = __float_as_uint(se[k]);
             }
             __syncthreads();
-            if (tid < TC && c0 + seg_at<VEC>(tid) < d && n > 0) {
+            if (tid < TC && c0 + seg_at<W>(tid) < d && n > 0) {
                 float a = 0.f, ae = 0.f;
                 for (int u = 0; u < kWarps; ++u) {
                     float ns, ne;
@@ -556,7 +580,7 @@ sweep_kernel(const SweepArgs A)
                     a = ns;
                     ae += ne + __uint_as_float(list[(2 * u + 1) * TC + tid]);
                 }
-                A.out[c0 + seg_at<VEC>(tid)] = (float)(((double)a + (double)ae) / (double)n);
+                A.out[c0 + seg_at<W>(tid)] = (float)(((double)a + (double)ae) / (double)n);
             }
             __syncthreads();
         } else {
@@ -611,7 +635,7 @@ sweep_kernel(const SweepArgs A)
                                 isfinite(cc);
                 S(S_VS, c) = __float_as_uint(ok ? sc : 0.f);
                 S(S_VC, c) = __float_as_uint(ok ? cc : 0.f);
-                S(S_BIN, c) = c0 + seg_at<VEC>(c) < d && n > 0 ? kLive | (ok ? 0u : 0xFFu) : 0u;
+                S(S_BIN, c) = c0 + seg_at<W>(c) < d && n > 0 ? kLive | (ok ? 0u : 0xFFu) : 0u;
             }
             __syncthreads();                                        // (B)
             const float4 vs = *reinterpret_cast<const float4 *>(&S(S_VS, lane * 4));
@@ -697,14 +721,14 @@ sweep_kernel(const SweepArgs A)
                         f2 |= hit;
                     }
                     // an overflowed counter or a NaN changes the coordinate's total
-                    if (tot == (uint32_t)n && cnt <= (uint32_t)kCap) {
+                    if (tot == (uint32_t)n && cnt <= cap) {
                         word = bin | kListed;
                         pend = cnt | (rem << 8);
                         if (cnt > (uint32_t)kShort) long_c[atomicAdd(&n_long[par], 1)] = (uint8_t)c;
                     }
                 }
                 if (state != 0u && word == 0u) {                    // left to fixup_kernel
-                    A.out[c0 + seg_at<VEC>(c)] = __uint_as_float(kOpen);
+                    A.out[c0 + seg_at<W>(c)] = __uint_as_float(kOpen);
                     ++open_cnt;
                 }
                 S(S_BIN, c) = word;
@@ -740,7 +764,7 @@ sweep_kernel(const SweepArgs A)
                             if (!(k == 0 ? m0 : k == 1 ? m1 : k == 2 ? m2 : m3)) continue;
                             const int c = lane * 4 + k;
                             const uint32_t at = atomicAdd(&S(S_LCNT, c), 1u);
-                            if (at < (uint32_t)kCap) list[at * TC + c] = el(v, k);
+                            if (at < cap) list[at * TC + c] = el(v, k);
                         }
                     }
                 };
@@ -787,11 +811,11 @@ sweep_kernel(const SweepArgs A)
                         const int b = __ffs(m) - 1;
                         const int k = b >> 3, j = g + (b & 7), c = lane * 4 + k;
                         const uint32_t at = atomicAdd(&S(S_LCNT, c), 1u);
-                        if (at < (uint32_t)kCap)
+                        if (at < cap)
                             cp_async4(list_s + (at * TC + c) * 4u,
                                       AVG ? reinterpret_cast<const char *>(A.means + (int64_t)(word_of(j) >> 16) * A.ldm +
                                                                            c0 + c)
-                                          : file_at(lb, j) + (uint64_t)slot_of(j) * ldb + (VEC ? k : 32 * k) * 4);
+                                          : file_at(lb, j) + (uint64_t)slot_of(j) * ldb + off_of<W>(k) * 4);
                     }
                 }
                 cp_async_commit();
@@ -825,13 +849,13 @@ sweep_kernel(const SweepArgs A)
     }
 }
 
-template <int R, bool VEC, int MODE, int MINB, bool AVG = false>
+template <int R, int W, int MODE, int MINB, bool AVG = false, int CAP = 32>
 cudaError_t try_sweep(bool &ok, const SweepArgs &A, cudaStream_t stream)
 {
     ok = false;
-    const SweepLayout L = sweep_layout<MODE>(A.f);
+    const SweepLayout L = sweep_layout<MODE, CAP>(A.f);
     if (L.total > smem_cap()) return cudaSuccess;
-    auto kern = sweep_kernel<R, VEC, MODE, MINB, AVG>;
+    auto kern = sweep_kernel<R, W, MODE, MINB, AVG, CAP>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
@@ -846,30 +870,36 @@ cudaError_t try_sweep(bool &ok, const SweepArgs &A, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-template <int R, bool VEC>
+template <int R, int W>
 cudaError_t sweep_for(bool &ok, const SweepArgs &A, int mode, cudaStream_t stream)
 {
     ok = false;
-    if (mode == 1) return try_sweep<R, VEC, MEAN, 2>(ok, A, stream);
+    if (mode == 1) return try_sweep<R, W, MEAN, 2>(ok, A, stream);
     // One block alone on its SM has more rows in flight: taken where the tags
     // leave no room for a second one, and where there are no more tiles than
     // SMs anyway.
     const bool alone = (A.d + TC - 1) / TC <= sm_count();
     cudaError_t e = cudaSuccess;
     if (A.f <= kTagFiles) {
-        if (!alone) e = try_sweep<R, VEC, TAGGED, 2>(ok, A, stream);
-        if (e == cudaSuccess && !ok) e = try_sweep<R, VEC, TAGGED, 1>(ok, A, stream);
+        if (!alone && A.f <= kPairFiles) {
+            e = try_sweep<R, W, TAGGED, 2>(ok, A, stream);
+            if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 2, false, 16>(ok, A, stream);
+        }
+        if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 1>(ok, A, stream);
         if (e != cudaSuccess || ok) return e;
     }
-    return try_sweep<R, VEC, TWO_PASS, 2>(ok, A, stream);
+    return try_sweep<R, W, TWO_PASS, 2>(ok, A, stream);
 }
 
 }  // namespace
 
 template <int R>
-cudaError_t launch_sweep(bool &ok, const SweepArgs &A, int mode, bool vec, cudaStream_t stream)
+cudaError_t launch_sweep(bool &ok, const SweepArgs &A, int mode, cudaStream_t stream)
 {
-    return vec ? sweep_for<R, true>(ok, A, mode, stream) : sweep_for<R, false>(ok, A, mode, stream);
+    const uintptr_t p = (uintptr_t)A.copies;
+    if (p % 16 == 0 && A.ld % 4 == 0) return sweep_for<R, 4>(ok, A, mode, stream);
+    if (p % 8 == 0 && A.ld % 2 == 0) return sweep_for<R, 2>(ok, A, mode, stream);
+    return sweep_for<R, 1>(ok, A, mode, stream);
 }
 
 template <int R>
@@ -877,8 +907,8 @@ cudaError_t launch_sweep_averages(bool &ok, const SweepArgs &A, cudaStream_t str
 {
     ok = false;
     cudaError_t e = cudaSuccess;
-    if ((A.d + TC - 1) / TC > sm_count()) e = try_sweep<R, true, TAGGED, 2, true>(ok, A, stream);
-    if (e == cudaSuccess && !ok) e = try_sweep<R, true, TAGGED, 1, true>(ok, A, stream);
+    if ((A.d + TC - 1) / TC > sm_count()) e = try_sweep<R, 4, TAGGED, 2, true>(ok, A, stream);
+    if (e == cudaSuccess && !ok) e = try_sweep<R, 4, TAGGED, 1, true>(ok, A, stream);
     return e;
 }
 
