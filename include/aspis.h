@@ -232,8 +232,8 @@ aspis_status aspis_round(const float *copies, int64_t d, int64_t ld,
  * process.  Every call copies the assignment table (f*r bytes) from the
  * library's pageable host memory into the array on the stream, so the call
  * may return only after the work already queued on the stream has drained.
- * All calls share the array and its contents persist between calls (the
- * parts that must start at zero are cleared by each call): calls that may
+ * All calls share the array and its contents persist between calls (each
+ * call overwrites what it reads): calls that may
  * overlap on the GPU, e.g. on unordered streams, race and must not be
  * issued. */
 aspis_status aspis_round_static(const float *copies, int64_t d, int64_t ld,

@@ -11,25 +11,30 @@ namespace aspis {
 
 int sm_count()
 {
-    static std::mutex mu;
-    static int cached[64] = {0};
+    static std::atomic<int> cached[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
-    std::lock_guard<std::mutex> g(mu);
-    if (!cached[dev]) {
-        int n = 0;
+    int n = cached[dev].load(std::memory_order_relaxed);
+    if (!n) {
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        cached[dev] = n > 0 ? n : 1;
+        if (n < 1) n = 1;
+        cached[dev].store(n, std::memory_order_relaxed);
     }
-    return cached[dev];
+    return n;
 }
 
 size_t smem_cap()
 {
-    int dev = 0, cap = 0;
+    static std::atomic<int> cached[64] = {};
+    int dev = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (dev < 0 || dev >= 64) dev = 0;
+    int cap = cached[dev].load(std::memory_order_relaxed);
+    if (!cap) {
+        cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cached[dev].store(cap, std::memory_order_relaxed);
+    }
     return (size_t)cap - 1024;        // static shared memory and reserve
 }
 
@@ -116,8 +121,6 @@ bool copy_and_compare(const float *host, float *dev, int64_t d, int64_t ld,
         L.ready = true;
     }
     const int64_t f = a->f, r = a->r, row = r * ld;               // floats per file
-    if ((err = cudaMemsetAsync(file_neq, 0, sizeof(uint32_t) * (size_t)f, st)) != cudaSuccess)
-        return true;
     const int64_t per = (f + kPipeChunks - 1) / kPipeChunks;
     const float *src = static_cast<const float *>(at.devicePointer);
     for (int k = 0; k < kPipeChunks; ++k) {
@@ -244,8 +247,6 @@ extern "C" aspis_status aspis_check(const float *copies, int64_t d, int64_t ld,
     if ((s = check_copies(copies, d, ld, a)) != ASPIS_OK) return s;
     if (!file_neq || !adj) return ASPIS_E_INVAL;
     cudaStream_t st = (cudaStream_t)stream;
-    if (cudaMemsetAsync(file_neq, 0, sizeof(uint32_t) * (size_t)a->f, st) != cudaSuccess)
-        return ASPIS_E_CUDA;
     if ((s = cuda_status(launch_compare(copies, a->f, a->r, d, ld, file_neq, st))) != ASPIS_OK)
         return s;
     return cuda_status(launch_graph(file_neq, a->dev_file_workers, a->f, a->r, a->K, adj, st));
@@ -310,8 +311,6 @@ extern "C" aspis_status aspis_round(const float *copies, int64_t d, int64_t ld,
                                        file_neq, adj, det, sel, mode, out, (cudaStream_t)stream));
     if (s != ASPIS_OK || done) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    if (cudaMemsetAsync(file_neq, 0, sizeof(uint32_t) * (size_t)a->f, st) != cudaSuccess)
-        return ASPIS_E_CUDA;
     if ((s = cuda_status(launch_compare(copies, a->f, a->r, d, ld, file_neq, st))) != ASPIS_OK) return s;
     s = cuda_status(launch_decide(file_neq, a->dev_file_workers, a->f, a->r, a->K, adj, det, sel, st));
     if (s != ASPIS_OK) return s;

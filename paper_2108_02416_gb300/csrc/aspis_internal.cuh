@@ -4,11 +4,14 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "aspis.h"
 
 namespace aspis {
 
 // Launch helpers: enqueue on `stream`, return cudaGetLastError().
+// launch_compare overwrites file_neq entirely.
 cudaError_t launch_compare(const float *copies, int64_t f, int r, int64_t d,
                            int64_t ld, uint32_t *file_neq, cudaStream_t stream);
 cudaError_t launch_graph(const uint32_t *file_neq, const uint8_t *dev_file_workers,
@@ -46,8 +49,40 @@ cudaError_t launch_round_fused(bool &done, const float *copies, int64_t f, int r
 // Number of SMs of the current device (cached per device).
 int sm_count();
 
-// Dynamic shared memory a block may ask for on the current device.
+// Dynamic shared memory a block may ask for on the current device (cached).
 size_t smem_cap();
+
+// Blocks of one kernel that an SM holds, asked of the runtime once per device
+// and amount of dynamic shared memory (the last amount is kept, in one word, so
+// that threads cannot see half of another's answer).
+class Residency {
+public:
+    template <class K>
+    int blocks(K kernel, int threads, size_t smem)
+    {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (dev < 0 || dev >= 64) dev = 0;
+        const uint64_t known = last_[dev].load(std::memory_order_relaxed);
+        if ((known >> 8) == smem + 1) return (int)(known & 0xFFu);
+        // (always the same limit: another thread's call may need more than this one)
+        if (smem > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_cap()) !=
+                            cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        last_[dev].store(((uint64_t)(smem + 1) << 8) | (uint64_t)(n < 255 ? n : 255), std::memory_order_relaxed);
+        return n;
+    }
+
+private:
+    std::atomic<uint64_t> last_[64] = {};
+};
 
 __host__ __device__ inline int pair_count(int r) { return r * (r - 1) / 2; }
 

@@ -22,11 +22,28 @@ __device__ __forceinline__ uint32_t vdiff(const uint4 &a, const uint4 &b)
     return (a.x ^ b.x) | (a.y ^ b.y) | (a.z ^ b.z) | (a.w ^ b.w);
 }
 
-template <int R, int U>
+// Files of one work item each (d up to 4 kChunkVec): a block ORs its warps'
+// words and writes the file's, so nothing has to be cleared first.
+__device__ __forceinline__ void write_word(uint32_t neq, uint32_t *words, uint32_t *to)
+{
+    neq = __reduce_or_sync(0xffffffffu, neq);
+    if ((threadIdx.x & 31) == 0) words[threadIdx.x >> 5] = neq;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t all = 0u;
+#pragma unroll
+        for (int q = 0; q < kCmpThreads / 32; ++q) all |= words[q];
+        *to = all;
+    }
+    __syncthreads();
+}
+
+template <int R, int U, bool DIRECT>
 __global__ void __launch_bounds__(kCmpThreads)
 compare_vec_kernel(const float *__restrict__ copies, int64_t f, int64_t d, int64_t ld,
                    int64_t nvec, int64_t nchunks, uint32_t *__restrict__ file_neq)
 {
+    __shared__ uint32_t words[DIRECT ? kCmpThreads / 32 : 1];
     const int64_t ldv = ld >> 2;
     const uint4 *base = reinterpret_cast<const uint4 *>(copies);
     const int64_t items = f * nchunks;
@@ -70,17 +87,22 @@ compare_vec_kernel(const float *__restrict__ copies, int64_t f, int64_t d, int64
                 for (int t = s + 1; t < R; ++t, ++p)
                     neq |= (y[s] != y[t] ? 1u : 0u) << p;
         }
-        neq = __reduce_or_sync(0xffffffffu, neq);
-        if ((threadIdx.x & 31) == 0 && neq) atomicOr(&file_neq[i], neq);
+        if constexpr (DIRECT) {
+            write_word(neq, words, &file_neq[i]);
+        } else {
+            neq = __reduce_or_sync(0xffffffffu, neq);
+            if ((threadIdx.x & 31) == 0 && neq) atomicOr(&file_neq[i], neq);
+        }
     }
 }
 
 // 4-byte path for buffers that are not 16-byte aligned or have ld % 4 != 0.
-template <int R>
+template <int R, bool DIRECT>
 __global__ void __launch_bounds__(kCmpThreads)
 compare_scalar_kernel(const float *__restrict__ copies, int64_t f, int64_t d, int64_t ld,
                       int64_t nchunks, uint32_t *__restrict__ file_neq)
 {
+    __shared__ uint32_t words[DIRECT ? kCmpThreads / 32 : 1];
     const uint32_t *base = reinterpret_cast<const uint32_t *>(copies);
     const int64_t chunk = kChunkVec * 4;
     const int64_t items = f * nchunks;
@@ -102,8 +124,12 @@ compare_scalar_kernel(const float *__restrict__ copies, int64_t f, int64_t d, in
                 for (int t = s + 1; t < R; ++t, ++p)
                     neq |= (y[s] != y[t] ? 1u : 0u) << p;
         }
-        neq = __reduce_or_sync(0xffffffffu, neq);
-        if ((threadIdx.x & 31) == 0 && neq) atomicOr(&file_neq[i], neq);
+        if constexpr (DIRECT) {
+            write_word(neq, words, &file_neq[i]);
+        } else {
+            neq = __reduce_or_sync(0xffffffffu, neq);
+            if ((threadIdx.x & 31) == 0 && neq) atomicOr(&file_neq[i], neq);
+        }
     }
 }
 
@@ -127,22 +153,27 @@ graph_kernel(const uint32_t *__restrict__ file_neq, const uint8_t *__restrict__ 
     }
 }
 
+template <int R, int U, bool DIRECT>
+cudaError_t start_vec(const float *copies, int64_t f, int64_t d, int64_t ld, int64_t nvec, int64_t nchunks,
+                      uint32_t *file_neq, cudaStream_t stream)
+{
+    static Residency resident;
+    const int64_t most = (int64_t)sm_count() * resident.blocks(compare_vec_kernel<R, U, DIRECT>, kCmpThreads, 0);
+    const int64_t grid = most < f * nchunks ? most : f * nchunks;
+    compare_vec_kernel<R, U, DIRECT><<<(unsigned)grid, kCmpThreads, 0, stream>>>(copies, f, d, ld, nvec, nchunks,
+                                                                                 file_neq);
+    return cudaGetLastError();
+}
+
 template <int R, int U>
 cudaError_t launch_vec(const float *copies, int64_t f, int64_t d, int64_t ld,
                        uint32_t *file_neq, cudaStream_t stream)
 {
     const int64_t nvec = d >> 2;
-    int64_t nchunks = (nvec + kChunkVec - 1) / kChunkVec;
-    if (nchunks < 1) nchunks = 1;
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, compare_vec_kernel<R, U>,
-                                                  kCmpThreads, 0);
-    if (per_sm < 1) per_sm = 1;
-    int64_t grid = (int64_t)sm_count() * per_sm;
-    if (grid > f * nchunks) grid = f * nchunks;
-    compare_vec_kernel<R, U><<<(unsigned)grid, kCmpThreads, 0, stream>>>(
-        copies, f, d, ld, nvec, nchunks, file_neq);
-    return cudaGetLastError();
+    const int64_t nchunks = nvec > kChunkVec ? (nvec + kChunkVec - 1) / kChunkVec : 1;
+    if (nchunks == 1) return start_vec<R, U, true>(copies, f, d, ld, nvec, nchunks, file_neq, stream);
+    const cudaError_t e = cudaMemsetAsync(file_neq, 0, sizeof(uint32_t) * (size_t)f, stream);
+    return e != cudaSuccess ? e : start_vec<R, U, false>(copies, f, d, ld, nvec, nchunks, file_neq, stream);
 }
 
 template <int R>
@@ -150,12 +181,16 @@ cudaError_t launch_scalar(const float *copies, int64_t f, int64_t d, int64_t ld,
                           uint32_t *file_neq, cudaStream_t stream)
 {
     const int64_t chunk = kChunkVec * 4;
-    int64_t nchunks = (d + chunk - 1) / chunk;
-    if (nchunks < 1) nchunks = 1;
+    const int64_t nchunks = (d + chunk - 1) / chunk;
     int64_t grid = (int64_t)sm_count() * 8;
     if (grid > f * nchunks) grid = f * nchunks;
-    compare_scalar_kernel<R><<<(unsigned)grid, kCmpThreads, 0, stream>>>(
-        copies, f, d, ld, nchunks, file_neq);
+    if (nchunks == 1) {
+        compare_scalar_kernel<R, true><<<(unsigned)grid, kCmpThreads, 0, stream>>>(copies, f, d, ld, nchunks, file_neq);
+        return cudaGetLastError();
+    }
+    const cudaError_t e = cudaMemsetAsync(file_neq, 0, sizeof(uint32_t) * (size_t)f, stream);
+    if (e != cudaSuccess) return e;
+    compare_scalar_kernel<R, false><<<(unsigned)grid, kCmpThreads, 0, stream>>>(copies, f, d, ld, nchunks, file_neq);
     return cudaGetLastError();
 }
 

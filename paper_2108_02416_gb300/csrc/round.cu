@@ -329,8 +329,8 @@ cudaError_t fused(bool &done, const SweepArgs &A, const uint8_t *fw, int K, uint
     if (e != cudaSuccess) return e;
     decide_kernel<R, GUESS><<<1, kDecideThreads, 0, stream>>>(A.file_neq, fw, A.f, K, adj, A.det, sel);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    bool ok = false;
-    if ((e = launch_sweep<R>(ok, A, mode, stream)) != cudaSuccess) return e;
+    bool ok = false, open = false;
+    if ((e = launch_sweep<R>(ok, open, A, mode, stream)) != cudaSuccess) return e;
     if (!ok) return cudaErrorInvalidValue;
     decide_kernel<R, VERIFY><<<1, kDecideThreads, 0, stream>>>(A.file_neq, fw, A.f, K, adj, A.det, sel);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -358,11 +358,12 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, i
     // coordinates, against 28 at 2,024 files, d = 9,000) or two passes with
     // more rows in flight (165 against 126 us at 3,003 files).
     if (mode == 0 && f > kTagFiles && !gate) return launch_aggregate_many(copies, f, r, d, ld, sel, det, out, stream);
-    bool ok = false;
-    const cudaError_t e = launch_sweep<1>(ok, A, mode, stream);
+    bool ok = false, open = false;
+    const cudaError_t e = launch_sweep<1>(ok, open, A, mode, stream);
     if (e != cudaSuccess) return e;
     if (!ok) return cudaErrorInvalidValue;
-    return mode == 0 ? launch_fixup(A, stream) : cudaSuccess;
+    // (a repair that does not run has settled nothing of the one-pass sweep)
+    return open || (gate && mode == 0) ? launch_fixup(A, stream) : cudaSuccess;
 }
 
 cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld,

@@ -11,8 +11,8 @@
 // that loads the library until the process exits.  Every call shares it, so
 // calls that overlap on the GPU (different streams without ordering, or
 // several host threads) race on it; calls on one stream are ordered.  Its
-// contents carry over from the previous call: the mismatch words, the only
-// part that must start at zero, are cleared on the stream by every call.
+// contents carry over from the previous call; every call overwrites what it
+// reads.
 #include <mutex>
 
 #include "aspis_internal.cuh"
@@ -80,8 +80,6 @@ extern "C" aspis_status aspis_round_static(const float *copies, int64_t d, int64
     const int r = a->r;
     if (cudaMemcpyAsync(fw, a->file_workers, (size_t)(f * r), cudaMemcpyHostToDevice, st) !=
         cudaSuccess)
-        return ASPIS_E_CUDA;
-    if (cudaMemsetAsync(file_neq, 0, sizeof(uint32_t) * (size_t)f, st) != cudaSuccess)
         return ASPIS_E_CUDA;
     if (launch_compare(copies, f, r, d, ld, file_neq, st) != cudaSuccess) return ASPIS_E_CUDA;
     if (launch_graph(file_neq, fw, f, r, a->K, adj, st) != cudaSuccess) return ASPIS_E_CUDA;

@@ -219,15 +219,152 @@ __device__ __forceinline__ int warp_ranked(uint32_t a, uint32_t b, uint32_t cnt,
     return 0;
 }
 
+// The coordinates that a block left open (kOpen in its part of out), at the end
+// of its sweep, where there are so few tiles that fixup_kernel's launch would
+// cost more (27 -> 24 us at 35 files of three, d = 4,096).  In larger calls the
+// mere presence of this call costs the sweep 5 to 9%.  32 coordinates at a time.
+//   Few of them open: one after the other, the values spread over the block's
+//   threads and their keys selected bit by bit (a load latency and 32 block
+//   counts: 5 to 10 us).
+//   Else an 8-bit radix select of all 32 at once: four passes over the rows'
+//   128-byte segments.
+__device__ __noinline__ void settle_open(const SweepArgs &A, uint32_t *hist, const uint32_t *meta, int n,
+                                         int64_t t0, int64_t tstep)
+{
+    constexpr int kPer = (ASPIS_MAX_AGG_FILES + kNT - 1) / kNT, kFew = 6;
+    __shared__ uint32_t pre[32], rnk[32], open_s;
+    __shared__ int counts[2][kWarps];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const unsigned full = 0xffffffffu;
+    const uint32_t krank = (uint32_t)((n - 1) / 2);
+    // the i-th kept row, NULL: none
+    auto row_of = [&](int i) -> const uint32_t * {
+        return i < n ? reinterpret_cast<const uint32_t *>(A.copies) + (int64_t)meta[i] * A.ld : nullptr;
+    };
+    const int64_t groups = (A.d + 31) / 32;
+    for (int64_t g0 = t0 * (TC / 32); g0 < groups; g0 += tstep * (TC / 32))
+        for (int64_t g = g0; g < g0 + TC / 32 && g < groups; ++g) {
+            const int64_t c0 = g * 32;
+            if (w == 0) {
+                const uint32_t x = c0 + lane < A.d ? __ldcg(reinterpret_cast<const unsigned int *>(A.out) + c0 + lane) : 0u;
+                const uint32_t m = __ballot_sync(full, x == kOpen);
+                if (lane == 0) open_s = m;
+            }
+            __syncthreads();
+            uint32_t open = open_s;
+            __syncthreads();
+            if (!open) continue;
+            if (__popc(open) <= kFew) {
+                for (; open; open &= open - 1u) {
+                    const int64_t c = c0 + __ffs(open) - 1;
+                    uint32_t key[kPer], has = 0u;
+#pragma unroll
+                    for (int u = 0; u < kPer; ++u) {
+                        const uint32_t *row = row_of(tid + u * kNT);
+                        key[u] = row ? to_key(__ldcg(row + c)) : 0u;
+                        has |= (row ? 1u : 0u) << u;
+                    }
+                    uint32_t prefix = 0u, rk = krank;
+                    for (int b = 31; b >= 0; --b) {
+                        // keys that match the prefix above bit b and have bit b clear
+                        int below = 0;
+#pragma unroll
+                        for (int u = 0; u < kPer; ++u) below += ((has >> u) & 1u) && (key[u] >> b) == (prefix >> b);
+                        below = __reduce_add_sync(full, below);
+                        if (lane == 0) counts[b & 1][w] = below;
+                        __syncthreads();
+                        below = 0;
+#pragma unroll
+                        for (int q = 0; q < kWarps; ++q) below += counts[b & 1][q];
+                        if (rk >= (uint32_t)below) {
+                            rk -= (uint32_t)below;
+                            prefix |= 1u << b;
+                        }
+                    }
+                    __syncthreads();
+                    if (tid == 0) A.out[c] = __uint_as_float(from_key(prefix));
+                }
+                __syncthreads();
+                continue;
+            }
+            const bool live = c0 + lane < A.d;
+            if (tid < 32) {
+                pre[tid] = 0u;
+                rnk[tid] = krank;
+            }
+            for (int p = 0; p < 4; ++p) {
+                const int sh = 24 - 8 * p;
+                const uint32_t pmask = p == 0 ? 0u : 0xFFFFFFFFu << (32 - 8 * p);
+                for (int i = tid; i < 256 * 32; i += kNT) hist[i] = 0u;
+                __syncthreads();
+                const uint32_t want = pre[lane];
+                for (int j0 = w; j0 < n; j0 += kWarps * 8) {
+                    uint32_t v[8], has = 0u;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const uint32_t *row = live ? row_of(j0 + u * kWarps) : nullptr;
+                        v[u] = row ? __ldcg(row + c0 + lane) : 0u;
+                        has |= (row ? 1u : 0u) << u;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const uint32_t key = to_key(v[u]);
+                        if (((has >> u) & 1u) && (key & pmask) == want)
+                            atomicAdd(&hist[((key >> sh) & 0xFFu) * 32 + lane], 1u);
+                    }
+                }
+                __syncthreads();
+                // a warp settles a digit of a coordinate: a warp scan over the 256 counts
+                for (int cc = w; cc < 32; cc += kWarps) {
+                    uint32_t cb[8], sum = 0u;
+#pragma unroll
+                    for (int b = 0; b < 8; ++b) {
+                        cb[b] = hist[(lane * 8 + b) * 32 + cc];
+                        sum += cb[b];
+                    }
+                    uint32_t inc = sum;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t y = __shfl_up_sync(full, inc, o);
+                        if (lane >= o) inc += y;
+                    }
+                    const uint32_t rk = rnk[cc], exc = inc - sum;
+                    const bool mine = exc <= rk && rk < inc;
+                    uint32_t dig = 0u, r2 = rk - exc;
+                    bool hit = false;
+#pragma unroll
+                    for (int b = 0; b < 8; ++b) {
+                        if (!hit && r2 < cb[b]) {
+                            dig = (uint32_t)(lane * 8 + b);
+                            hit = true;
+                        }
+                        if (!hit) r2 -= cb[b];
+                    }
+                    const unsigned bal = __ballot_sync(full, mine);
+                    const int src = bal ? __ffs(bal) - 1 : 0;
+                    dig = __shfl_sync(full, dig, src);
+                    r2 = __shfl_sync(full, r2, src);
+                    if (lane == 0 && bal) {
+                        pre[cc] |= dig << sh;
+                        rnk[cc] = r2;
+                    }
+                }
+                __syncthreads();
+            }
+            if (w == 0 && ((open >> lane) & 1u)) A.out[c0 + lane] = __uint_as_float(from_key(pre[lane]));
+            __syncthreads();
+        }
+}
+
 // AVG: a file's value is the average of its copies in slot_mask; the meta word
 // holds the mask in place of slot and pair word.
-template <int R, int W, int MODE, int MINB, bool AVG, int CAP>
+template <int R, int W, int MODE, int MINB, bool AVG, int CAP, bool SETTLE>
 __global__ void __launch_bounds__(kNT, MINB)
 sweep_kernel(const SweepArgs A)
 {
     if (R == 1 && !gate_open(A.gate)) return;
     constexpr int kShort = MINB == 1 || (MODE == TWO_PASS && R == 1) ? 16 : 8;   // longest list one thread sorts
-    constexpr int kF = batch_files(R, MINB);
+    constexpr int kF = R == 1 && W == 4 && MODE == MEAN ? 6 : batch_files(R, MINB);
     constexpr int kRows = kF * R;
     static_assert(kF >= 2, "the sample is the first two files of every warp");
     extern __shared__ __align__(16) unsigned char smem[];
@@ -838,6 +975,9 @@ sweep_kernel(const SweepArgs A)
             open_cnt = __reduce_add_sync(full, open_cnt);
             if (lane == 0 && open_cnt) atomicAdd(&A.det->median_exact, open_cnt);
         }
+        if constexpr (SETTLE) {
+            if (__syncthreads_or(open_cnt != 0u)) settle_open(A, hist, meta, n, blockIdx.x, gridDim.x);
+        }
     }
     if constexpr (R == 1) {
         if (tid == 0) gate_leave(A.gate);
@@ -849,18 +989,15 @@ sweep_kernel(const SweepArgs A)
     }
 }
 
-template <int R, int W, int MODE, int MINB, bool AVG = false, int CAP = 32>
+template <int R, int W, int MODE, int MINB, bool AVG = false, int CAP = 32, bool SETTLE = false>
 cudaError_t try_sweep(bool &ok, const SweepArgs &A, cudaStream_t stream)
 {
     ok = false;
     const SweepLayout L = sweep_layout<MODE, CAP>(A.f);
     if (L.total > smem_cap()) return cudaSuccess;
-    auto kern = sweep_kernel<R, W, MODE, MINB, AVG, CAP>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kNT, L.total);
-    if (e != cudaSuccess) return e;
+    auto kern = sweep_kernel<R, W, MODE, MINB, AVG, CAP, SETTLE>;
+    static Residency resident;
+    const int per_sm = resident.blocks(kern, kNT, L.total);
     if (per_sm < MINB) return cudaSuccess;                // the next configuration is tried
     const int64_t ntiles = (A.d + TC - 1) / TC;
     int64_t grid = (int64_t)sm_count() * per_sm;
@@ -871,8 +1008,9 @@ cudaError_t try_sweep(bool &ok, const SweepArgs &A, cudaStream_t stream)
 }
 
 template <int R, int W>
-cudaError_t sweep_for(bool &ok, const SweepArgs &A, int mode, cudaStream_t stream)
+cudaError_t sweep_for(bool &ok, bool &open, const SweepArgs &A, int mode, cudaStream_t stream)
 {
+    open = mode == 0;
     ok = false;
     if (mode == 1) return try_sweep<R, W, MEAN, 2>(ok, A, stream);
     // One block alone on its SM has more rows in flight: taken where the tags
@@ -880,6 +1018,13 @@ cudaError_t sweep_for(bool &ok, const SweepArgs &A, int mode, cudaStream_t strea
     // SMs anyway.
     const bool alone = (A.d + TC - 1) / TC <= sm_count();
     cudaError_t e = cudaSuccess;
+    if constexpr (R == 1) {
+        if (alone && A.f <= kTagFiles) {
+            e = try_sweep<R, W, TAGGED, 1, false, 32, true>(ok, A, stream);
+            if (ok) open = false;
+            return e;
+        }
+    }
     if (A.f <= kTagFiles) {
         if (!alone && A.f <= kPairFiles) {
             e = try_sweep<R, W, TAGGED, 2>(ok, A, stream);
@@ -894,12 +1039,12 @@ cudaError_t sweep_for(bool &ok, const SweepArgs &A, int mode, cudaStream_t strea
 }  // namespace
 
 template <int R>
-cudaError_t launch_sweep(bool &ok, const SweepArgs &A, int mode, cudaStream_t stream)
+cudaError_t launch_sweep(bool &ok, bool &open, const SweepArgs &A, int mode, cudaStream_t stream)
 {
     const uintptr_t p = (uintptr_t)A.copies;
-    if (p % 16 == 0 && A.ld % 4 == 0) return sweep_for<R, 4>(ok, A, mode, stream);
-    if (p % 8 == 0 && A.ld % 2 == 0) return sweep_for<R, 2>(ok, A, mode, stream);
-    return sweep_for<R, 1>(ok, A, mode, stream);
+    if (p % 16 == 0 && A.ld % 4 == 0) return sweep_for<R, 4>(ok, open, A, mode, stream);
+    if (p % 8 == 0 && A.ld % 2 == 0) return sweep_for<R, 2>(ok, open, A, mode, stream);
+    return sweep_for<R, 1>(ok, open, A, mode, stream);
 }
 
 template <int R>
