@@ -314,7 +314,7 @@ extern "C" aspis_status aspis_round(const float *copies, int64_t d, int64_t ld,
     if ((s = cuda_status(launch_compare(copies, a->f, a->r, d, ld, file_neq, st))) != ASPIS_OK) return s;
     s = cuda_status(launch_decide(file_neq, a->dev_file_workers, a->f, a->r, a->K, adj, det, sel, st));
     if (s != ASPIS_OK) return s;
-    return aspis_aggregate(copies, d, ld, a, sel, det, mode, out, stream);
+    return cuda_status(launch_aggregate(copies, a->f, a->r, d, ld, sel, det, mode, out, st, nullptr, true));
 }
 
 extern "C" aspis_status aspis_round_host(const float *host_copies, float *dev_copies,

@@ -44,6 +44,7 @@ compare_vec_kernel(const float *__restrict__ copies, int64_t f, int64_t d, int64
                    int64_t nvec, int64_t nchunks, uint32_t *__restrict__ file_neq)
 {
     __shared__ uint32_t words[DIRECT ? kCmpThreads / 32 : 1];
+    chain();
     const int64_t ldv = ld >> 2;
     const uint4 *base = reinterpret_cast<const uint4 *>(copies);
     const int64_t items = f * nchunks;
@@ -103,6 +104,7 @@ compare_scalar_kernel(const float *__restrict__ copies, int64_t f, int64_t d, in
                       int64_t nchunks, uint32_t *__restrict__ file_neq)
 {
     __shared__ uint32_t words[DIRECT ? kCmpThreads / 32 : 1];
+    chain();
     const uint32_t *base = reinterpret_cast<const uint32_t *>(copies);
     const int64_t chunk = kChunkVec * 4;
     const int64_t items = f * nchunks;

@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(kSampleThreads)
 sample_kernel(const uint32_t *__restrict__ copies, int64_t f, int64_t d, int64_t ld,
               uint32_t *__restrict__ file_neq)
 {
+    chain();
     const int lane = threadIdx.x & 31;
     const int64_t i = (int64_t)blockIdx.x * (kSampleThreads / 32) + (threadIdx.x >> 5);
     if (i >= f) return;
@@ -92,6 +93,7 @@ decide_kernel(uint32_t *__restrict__ file_neq, const uint8_t *__restrict__ fw, i
     __shared__ Frame stack[32][32];
     __shared__ int best, kept, success_s;
     __shared__ uint32_t clique_s;
+    chain();
     const int tid = threadIdx.x;
     if (tid < 32) dis[tid] = 0u;
     if (tid == 0) {
@@ -166,6 +168,7 @@ static_assert(kFixPer * kFixThreads == ASPIS_MAX_AGG_FILES, "every kept value ha
 __global__ void __launch_bounds__(kFixThreads)
 fixup_kernel(const SweepArgs A)
 {
+    chain();
     if (*(volatile const uint32_t *)&A.det->median_exact == 0u) return;
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t *hist = reinterpret_cast<uint32_t *>(smem);              // [256][32]
@@ -315,8 +318,7 @@ cudaError_t launch_fixup(const SweepArgs &A, cudaStream_t stream)
     const int64_t ntiles = (A.d + 31) / 32;
     int64_t grid = (int64_t)sm_count() * 4;
     if (grid > ntiles) grid = ntiles;
-    fixup_kernel<<<(unsigned)grid, kFixThreads, smem, stream>>>(A);
-    return cudaGetLastError();
+    return launch_chained(fixup_kernel, grid, kFixThreads, smem, stream, A);
 }
 
 template <int R>
@@ -327,30 +329,29 @@ cudaError_t fused(bool &done, const SweepArgs &A, const uint8_t *fw, int K, uint
         reinterpret_cast<const uint32_t *>(A.copies), A.f, A.d, A.ld, A.file_neq);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    decide_kernel<R, GUESS><<<1, kDecideThreads, 0, stream>>>(A.file_neq, fw, A.f, K, adj, A.det, sel);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_chained(decide_kernel<R, GUESS>, 1, kDecideThreads, 0, stream, A.file_neq, fw, A.f, K, adj, A.det, sel);
+    if (e != cudaSuccess) return e;
     bool ok = false, open = false;
-    if ((e = launch_sweep<R>(ok, open, A, mode, stream)) != cudaSuccess) return e;
+    if ((e = launch_sweep<R>(ok, open, A, mode, true, stream)) != cudaSuccess) return e;
     if (!ok) return cudaErrorInvalidValue;
-    decide_kernel<R, VERIFY><<<1, kDecideThreads, 0, stream>>>(A.file_neq, fw, A.f, K, adj, A.det, sel);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    e = launch_chained(decide_kernel<R, VERIFY>, 1, kDecideThreads, 0, stream, A.file_neq, fw, A.f, K, adj, A.det, sel);
+    if (e != cudaSuccess) return e;
     done = true;
-    return launch_aggregate(A.copies, A.f, R, A.d, A.ld, sel, A.det, mode, A.out, stream, A.det);
+    return launch_aggregate(A.copies, A.f, R, A.d, A.ld, sel, A.det, mode, A.out, stream, A.det, true);
 }
 
 template <int R>
 cudaError_t decide(uint32_t *file_neq, const uint8_t *fw, int f, int K, uint32_t *adj, aspis_detection *det,
                    int8_t *sel, cudaStream_t stream)
 {
-    decide_kernel<R, PLAIN><<<1, kDecideThreads, 0, stream>>>(file_neq, fw, f, K, adj, det, sel);
-    return cudaGetLastError();
+    return launch_chained(decide_kernel<R, PLAIN>, 1, kDecideThreads, 0, stream, file_neq, fw, f, K, adj, det, sel);
 }
 
 }  // namespace
 
 cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, int64_t ld, const int8_t *sel,
                              aspis_detection *det, int mode, float *out, cudaStream_t stream,
-                             aspis_detection *gate)
+                             aspis_detection *gate, bool chained)
 {
     if (f > ASPIS_MAX_AGG_FILES || f * r > 65535) return cudaErrorInvalidValue;
     const SweepArgs A{copies, d, ld, (int)f, sel, det, out, nullptr, r, gate, nullptr, nullptr, 0};
@@ -359,7 +360,7 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, i
     // more rows in flight (165 against 126 us at 3,003 files).
     if (mode == 0 && f > kTagFiles && !gate) return launch_aggregate_many(copies, f, r, d, ld, sel, det, out, stream);
     bool ok = false, open = false;
-    const cudaError_t e = launch_sweep<1>(ok, open, A, mode, stream);
+    const cudaError_t e = launch_sweep<1>(ok, open, A, mode, chained, stream);
     if (e != cudaSuccess) return e;
     if (!ok) return cudaErrorInvalidValue;
     // (a repair that does not run has settled nothing of the one-pass sweep)

@@ -53,7 +53,7 @@ struct SweepArgs {
 
 // ok = false where no layout holds f files; open = fixup_kernel has to follow.
 template <int R>
-cudaError_t launch_sweep(bool &ok, bool &open, const SweepArgs &A, int mode, cudaStream_t stream);
+cudaError_t launch_sweep(bool &ok, bool &open, const SweepArgs &A, int mode, bool chained, cudaStream_t stream);
 
 // The median of the averages of the copies in slot_mask, which are also written
 // to means (R > 1, aligned rows, f <= kTagFiles); nothing is compared.

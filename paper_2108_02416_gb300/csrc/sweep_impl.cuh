@@ -362,6 +362,7 @@ template <int R, int W, int MODE, int MINB, bool AVG, int CAP, bool SETTLE>
 __global__ void __launch_bounds__(kNT, MINB)
 sweep_kernel(const SweepArgs A)
 {
+    chain();
     if (R == 1 && !gate_open(A.gate)) return;
     constexpr int kShort = MINB == 1 || (MODE == TWO_PASS && R == 1) ? 16 : 8;   // longest list one thread sorts
     constexpr int kF = R == 1 && W == 4 && MODE == MEAN ? 6 : batch_files(R, MINB);
@@ -990,7 +991,7 @@ sweep_kernel(const SweepArgs A)
 }
 
 template <int R, int W, int MODE, int MINB, bool AVG = false, int CAP = 32, bool SETTLE = false>
-cudaError_t try_sweep(bool &ok, const SweepArgs &A, cudaStream_t stream)
+cudaError_t try_sweep(bool &ok, const SweepArgs &A, bool chained, cudaStream_t stream)
 {
     ok = false;
     const SweepLayout L = sweep_layout<MODE, CAP>(A.f);
@@ -1002,17 +1003,18 @@ cudaError_t try_sweep(bool &ok, const SweepArgs &A, cudaStream_t stream)
     const int64_t ntiles = (A.d + TC - 1) / TC;
     int64_t grid = (int64_t)sm_count() * per_sm;
     if (grid > ntiles) grid = ntiles;
-    kern<<<(unsigned)grid, kNT, L.total, stream>>>(A);
     ok = true;
+    if (chained) return launch_chained(kern, grid, kNT, L.total, stream, A);
+    kern<<<(unsigned)grid, kNT, L.total, stream>>>(A);
     return cudaGetLastError();
 }
 
 template <int R, int W>
-cudaError_t sweep_for(bool &ok, bool &open, const SweepArgs &A, int mode, cudaStream_t stream)
+cudaError_t sweep_for(bool &ok, bool &open, const SweepArgs &A, int mode, bool chained, cudaStream_t stream)
 {
     open = mode == 0;
     ok = false;
-    if (mode == 1) return try_sweep<R, W, MEAN, 2>(ok, A, stream);
+    if (mode == 1) return try_sweep<R, W, MEAN, 2>(ok, A, chained, stream);
     // One block alone on its SM has more rows in flight: taken where the tags
     // leave no room for a second one, and where there are no more tiles than
     // SMs anyway.
@@ -1020,40 +1022,41 @@ cudaError_t sweep_for(bool &ok, bool &open, const SweepArgs &A, int mode, cudaSt
     cudaError_t e = cudaSuccess;
     if constexpr (R == 1) {
         if (alone && A.f <= kTagFiles) {
-            e = try_sweep<R, W, TAGGED, 1, false, 32, true>(ok, A, stream);
+            e = try_sweep<R, W, TAGGED, 1, false, 32, true>(ok, A, chained, stream);
             if (ok) open = false;
             return e;
         }
     }
     if (A.f <= kTagFiles) {
         if (!alone && A.f <= kPairFiles) {
-            e = try_sweep<R, W, TAGGED, 2>(ok, A, stream);
-            if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 2, false, 16>(ok, A, stream);
+            e = try_sweep<R, W, TAGGED, 2>(ok, A, chained, stream);
+            if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 2, false, 16>(ok, A, chained, stream);
         }
-        if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 1>(ok, A, stream);
+        if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 1>(ok, A, chained, stream);
         if (e != cudaSuccess || ok) return e;
     }
-    return try_sweep<R, W, TWO_PASS, 2>(ok, A, stream);
+    return try_sweep<R, W, TWO_PASS, 2>(ok, A, chained, stream);
 }
 
 }  // namespace
 
 template <int R>
-cudaError_t launch_sweep(bool &ok, bool &open, const SweepArgs &A, int mode, cudaStream_t stream)
+cudaError_t launch_sweep(bool &ok, bool &open, const SweepArgs &A, int mode, bool chained, cudaStream_t stream)
 {
     const uintptr_t p = (uintptr_t)A.copies;
-    if (p % 16 == 0 && A.ld % 4 == 0) return sweep_for<R, 4>(ok, open, A, mode, stream);
-    if (p % 8 == 0 && A.ld % 2 == 0) return sweep_for<R, 2>(ok, open, A, mode, stream);
-    return sweep_for<R, 1>(ok, open, A, mode, stream);
+    if (p % 16 == 0 && A.ld % 4 == 0) return sweep_for<R, 4>(ok, open, A, mode, chained, stream);
+    if (p % 8 == 0 && A.ld % 2 == 0) return sweep_for<R, 2>(ok, open, A, mode, chained, stream);
+    return sweep_for<R, 1>(ok, open, A, mode, chained, stream);
 }
 
 template <int R>
 cudaError_t launch_sweep_averages(bool &ok, const SweepArgs &A, cudaStream_t stream)
 {
     ok = false;
+    const bool chained = false;
     cudaError_t e = cudaSuccess;
-    if ((A.d + TC - 1) / TC > sm_count()) e = try_sweep<R, 4, TAGGED, 2, true>(ok, A, stream);
-    if (e == cudaSuccess && !ok) e = try_sweep<R, 4, TAGGED, 1, true>(ok, A, stream);
+    if ((A.d + TC - 1) / TC > sm_count()) e = try_sweep<R, 4, TAGGED, 2, true>(ok, A, chained, stream);
+    if (e == cudaSuccess && !ok) e = try_sweep<R, 4, TAGGED, 1, true>(ok, A, chained, stream);
     return e;
 }
 

@@ -2,5 +2,5 @@
 #include "sweep_impl.cuh"
 
 namespace aspis {
-template cudaError_t launch_sweep<1>(bool &, bool &, const SweepArgs &, int, cudaStream_t);
+template cudaError_t launch_sweep<1>(bool &, bool &, const SweepArgs &, int, bool, cudaStream_t);
 }  // namespace aspis

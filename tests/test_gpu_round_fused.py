@@ -133,3 +133,45 @@ def test_guess_of_an_earlier_round_is_not_kept():
         ap.aspis_round(torch.from_numpy(host).to(DEV), d, a, buf.file_neq, buf.adj, buf.det, buf.sel, buf.out)
         torch.cuda.synchronize()
         assert_round_matches(ap, buf, want)
+
+
+@pytest.mark.parametrize("K,r,d", [(7, 3, 4099), (15, 3, 36_933), (15, 3, 190_001)])
+def test_rounds_back_to_back_captured_and_on_two_streams(K, r, d):
+    """Kernels of one round overlap their launches: nothing may run ahead of
+    the round before it on the stream, in a graph, or beside another stream."""
+    a = ap.aspis_assign(K, r)
+    rounds = []
+    for seed, attack in ((1, "weak"), (2, "strong")):
+        oa, host, mask = build(K, r, d, 2, attack, seed, ld=(d + 3) // 4 * 4)
+        host[mask] += np.float32(1.0)
+        rounds.append((torch.from_numpy(host).to(DEV), ap.RoundBuffers(a, d, DEV), oracle.run_round(host, oa, d, 0)))
+
+    def one(k, buf, stream=None):
+        ap.aspis_round(rounds[k][0], d, a, buf.file_neq, buf.adj, buf.det, buf.sel, buf.out, ap.MEDIAN, stream)
+
+    shared = ap.RoundBuffers(a, d, DEV)
+    for last in (0, 1):
+        for k in (0, 1, 1, 0, 1 - last, last):
+            one(k, shared)
+        torch.cuda.synchronize()
+        assert_round_matches(ap, shared, rounds[last][2])
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for k in (0, 1):
+            one(k, rounds[k][1], torch.cuda.current_stream())
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    for k in (0, 1):
+        assert_round_matches(ap, rounds[k][1], rounds[k][2])
+        rounds[k][1].out.zero_()
+
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    for _ in range(5):
+        for k in (0, 1):
+            one(k, rounds[k][1], streams[k])
+    torch.cuda.synchronize()
+    for k in (0, 1):
+        assert_round_matches(ap, rounds[k][1], rounds[k][2])
