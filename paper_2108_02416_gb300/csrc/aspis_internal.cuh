@@ -36,6 +36,9 @@ cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, in
 // The lower median for f > kTagFiles (aggregate.cu).
 cudaError_t launch_aggregate_many(const float *copies, int64_t f, int r, int64_t d, int64_t ld,
                                   const int8_t *sel, aspis_detection *det, float *out, cudaStream_t stream);
+// At most kFewFiles files (sweep.cuh), median.
+cudaError_t launch_aggregate_few(const float *copies, int64_t f, int r, int64_t d, int64_t ld, const int8_t *sel,
+                                 aspis_detection *det, float *out, bool chained, cudaStream_t stream);
 // Steps 2-4 (graph, maximum cliques, selection) in one launch, for f <=
 // ASPIS_MAX_AGG_FILES.
 cudaError_t launch_decide(uint32_t *file_neq, const uint8_t *dev_file_workers, int64_t f, int r, int K,
@@ -58,9 +61,9 @@ size_t smem_cap();
 // wait in chain() for its end and its writes, which hides the 2 to 3 us between
 // dependent kernels.  Every kernel of a chain calls chain() before it touches
 // global memory; the first one is launched plainly, and so waits for all earlier
-// work on the stream.  Measured: the six kernels over 455 files of three and
-// d = 36,932 65 us against 72, the three over 35 files and d = 4,096 21.3 against
-// 23.3, the six at d = 1,048,576 1,222 against 1,225.
+// work on the stream.  Measured: the separate kernels of a round over 455 files
+// of three and d = 36,932 65 us against 72, over 35 files and d = 4,096 21.3 against
+// 23.3, the six of the one-pass round at d = 1,048,576 1,222 against 1,225.
 __device__ __forceinline__ void chain()
 {
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");

@@ -3,6 +3,8 @@
 // search modes of the lower median.
 #pragma once
 
+#include <utility>
+
 #include <stdint.h>
 
 namespace aspis {
@@ -157,6 +159,52 @@ __device__ __forceinline__ float mean_masked(const float (&x)[R], uint32_t m, in
             acc = __fadd_rn(acc, e);
         }
     return acc == 0.f ? x0 : __fadd_rn(x0, __fdiv_rn(acc, (float)k));
+}
+
+// Ascending odd-even merge sort of N <= 64 keys in registers (Batcher 1968):
+// the comparators of the 32-key (64-key) network, those that touch a key beyond
+// N dropped (they would meet the largest key).
+struct Network {
+    int n = 0;
+    unsigned char a[544] = {}, b[544] = {};
+};
+
+template <int N>
+__host__ __device__ constexpr Network merge_network()
+{
+    constexpr int kWide = N <= 32 ? 32 : 64;
+    Network net{};
+    for (int p = 1; p < kWide; p *= 2)
+        for (int k = p; k >= 1; k /= 2)
+            for (int j = k % p; j + k < kWide; j += 2 * k)
+                for (int i = 0; i < k; ++i)
+                    if (i + j + k < N && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
+                        net.a[net.n] = (unsigned char)(i + j);
+                        net.b[net.n] = (unsigned char)(i + j + k);
+                        ++net.n;
+                    }
+    return net;
+}
+
+template <int A, int B, int N>
+__device__ __forceinline__ void compare_exchange(uint32_t (&y)[N])
+{
+    const uint32_t a = y[A], b = y[B];
+    y[A] = min(a, b);
+    y[B] = max(a, b);
+}
+
+template <int N, int... I>
+__device__ __forceinline__ void merge_sort(uint32_t (&y)[N], std::integer_sequence<int, I...>)
+{
+    constexpr Network net = merge_network<N>();
+    (compare_exchange<net.a[I], net.b[I]>(y), ...);
+}
+
+template <int N>
+__device__ __forceinline__ void merge_sort(uint32_t (&y)[N])
+{
+    merge_sort<N>(y, std::make_integer_sequence<int, merge_network<N>().n>{});
 }
 
 }  // namespace aspis

@@ -355,6 +355,9 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, i
 {
     if (f > ASPIS_MAX_AGG_FILES || f * r > 65535) return cudaErrorInvalidValue;
     const SweepArgs A{copies, d, ld, (int)f, sel, det, out, nullptr, r, gate, nullptr, nullptr, 0};
+    // Few files: whole values sorted in registers (89 us for the round against 52 at
+    // 35 files of three, d = 400,000; 24 against 23 at 4,096).
+    if (mode == 0 && f <= kFewFiles && !gate) return launch_aggregate_few(copies, f, r, d, ld, sel, det, out, chained, stream);
     // Many files: one pass over narrow tiles (92 us, and 28 more for the open
     // coordinates, against 28 at 2,024 files, d = 9,000) or two passes with
     // more rows in flight (165 against 126 us at 3,003 files).
@@ -373,8 +376,9 @@ cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, in
 {
     done = false;
     // (62 against 54 us at 455 files of three and d = 4,096, 73 against 75 at
-    // 16,384, 176 against 199 at 65,536)
-    if (r > 5 || f > kTagFiles || f * r * d < kMinAverages) return cudaSuccess;
+    // 16,384, 176 against 199 at 65,536; with few files the tiles' fixed work costs
+    // more than reading the averages again: 1,079 against 786 us at 35 and 4,000,000)
+    if (r > 5 || f <= kFewFiles || f > kTagFiles || f * r * d < kMinAverages) return cudaSuccess;
     const SweepArgs A{copies, d, ld, (int)f, sel, det, out, nullptr, r, nullptr, slot_mask, means, ldm};
     cudaError_t e;
     switch (r) {
@@ -400,6 +404,9 @@ cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, in
 // on 304 blocks, 1,309 against 1,355 with 1,024.
 bool one_pass_pays(int64_t f, int r, int64_t d, int mode)
 {
+    // few files (35 of three, d = 11,173,962): 1,223 us apart, 1,332 with the copies
+    // compared and sorted in registers in one pass, 1,736 with the tile kernel
+    if (mode == 0 && f <= kFewFiles) return false;
     const bool many = mode == 0 && f > kTagFiles;                       // two passes over the chosen rows
     if (f * r * d < (many ? 10 : 1) * kMinValues) return false;
     const int64_t tiles = (d + 127) / 128;

@@ -22,8 +22,6 @@
 // against 6.2 ms at 3,003 files of five copies and d = 2^19.)
 #pragma once
 
-#include <utility>
-
 #include "aspis_internal.cuh"
 #include "median_common.cuh"
 
@@ -31,6 +29,7 @@ namespace aspis {
 
 constexpr int64_t kPairFiles = 516;         // most files whose tag bytes let two blocks share an SM
 constexpr int64_t kTagFiles = 1330;         // most files whose tag bytes leave a tile room in a block
+constexpr int kFewFiles = 36;               // most files whose values one thread sorts in registers (few.cu)
 constexpr int kUnclean = 16;                // in a guessed sel: copies of the file differ
 // Bits of a coordinate that the sweep leaves to fixup_kernel.  They may also
 // be a median's own bits (a NaN payload): computing that one again gives it.

@@ -123,51 +123,6 @@ __device__ __forceinline__ uint32_t vdiff(const uint4 &a, const uint4 &b)
     return (a.x ^ b.x) | (a.y ^ b.y) | (a.z ^ b.z) | (a.w ^ b.w);
 }
 
-// Ascending odd-even merge sort of N <= 32 keys in registers (Batcher 1968):
-// the comparators of the 32-key network, those that touch a key beyond N
-// dropped (they would meet the largest key).
-struct Network {
-    int n = 0;
-    unsigned char a[192] = {}, b[192] = {};
-};
-
-template <int N>
-__host__ __device__ constexpr Network merge_network()
-{
-    Network net{};
-    for (int p = 1; p < 32; p *= 2)
-        for (int k = p; k >= 1; k /= 2)
-            for (int j = k % p; j + k < 32; j += 2 * k)
-                for (int i = 0; i < k; ++i)
-                    if (i + j + k < N && (i + j) / (2 * p) == (i + j + k) / (2 * p)) {
-                        net.a[net.n] = (unsigned char)(i + j);
-                        net.b[net.n] = (unsigned char)(i + j + k);
-                        ++net.n;
-                    }
-    return net;
-}
-
-template <int A, int B, int N>
-__device__ __forceinline__ void compare_exchange(uint32_t (&y)[N])
-{
-    const uint32_t a = y[A], b = y[B];
-    y[A] = min(a, b);
-    y[B] = max(a, b);
-}
-
-template <int N, int... I>
-__device__ __forceinline__ void merge_sort(uint32_t (&y)[N], std::integer_sequence<int, I...>)
-{
-    constexpr Network net = merge_network<N>();
-    (compare_exchange<net.a[I], net.b[I]>(y), ...);
-}
-
-template <int N>
-__device__ __forceinline__ void merge_sort(uint32_t (&y)[N])
-{
-    merge_sort<N>(y, std::make_integer_sequence<int, merge_network<N>().n>{});
-}
-
 // The file (a multiple of 8) that a tile's order starts from: its first kSample
 // files are the sample, so as few of them as possible shall be marked (bit 31:
 // their copies differ).  Neighbours in file order share workers, and with them

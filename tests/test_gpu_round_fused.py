@@ -175,3 +175,30 @@ def test_rounds_back_to_back_captured_and_on_two_streams(K, r, d):
     torch.cuda.synchronize()
     for k in (0, 1):
         assert_round_matches(ap, rounds[k][1], rounds[k][2])
+
+
+@pytest.mark.parametrize("K,r,d,attack", [(3, 2, 65, "weak"), (7, 3, 1, "strong"), (7, 3, 63, "weak"),
+                                          (7, 3, 19_521, "strong"), (9, 2, 4097, "weak"), (6, 4, 30_001, "strong"),
+                                          (6, 5, 64, "weak"), (7, 6, 4100, "weak")])
+@pytest.mark.parametrize("odd", [0, 1])
+def test_few_files(K, r, d, attack, odd):
+    """At most 36 files: sorted in registers, at any alignment, with values of
+    every kind (NaNs, infinities, zeros of both signs, the extreme keys)."""
+    oa, host, mask = build(K, r, d, 1, attack, 21, ld=d + 3 + odd)
+    f = oa.f
+    u = host.view(np.uint32)
+    for c, (a, b) in enumerate([(0xFFFFFFFF, 0x7FFFFFFF), (0x00000000, 0x80000000), (0xFF800000, 0x7F800000)]):
+        if c < d - 1:
+            u[:, :, c] = np.where(np.arange(f) % 2, a, b)[:, None]
+    host[mask] += np.float32(1e-3)
+    host[:, :, d:] = np.random.default_rng(3).standard_normal(host[:, :, d:].shape)
+    check(oa, host, d)
+
+
+def test_few_files_with_many_values():
+    """Few files never take the one-pass round: a length at which others do."""
+    d = smallest_d(7, 3) + 1
+    oa, host, mask = build(7, 3, d, 2, "strong", 5)
+    for i, s in zip(*np.nonzero(mask)):
+        host[i, s, d // 2 + 7 * i] += 5.0
+    check(oa, host, d)
