@@ -1,9 +1,11 @@
 """Benchmark of the Aspis PS detection-and-aggregation step on GB300.
 
-One step = one PS round on one GPU: aspis_check (compare every copy pair of
-every file, build G), aspis_detect (maximum cliques), aspis_select (one copy
-per file) and aspis_aggregate (coordinate-wise lower median), all on one
-stream, over synthetic copies already resident in HBM.
+One step = one PS round on one GPU, the public call aspis_round: compare every
+copy pair of every file, build G, find the maximum cliques, select one copy per
+file and take the coordinate-wise lower median, all on one stream, over
+synthetic copies already resident in HBM.  The same round through the separate
+calls (aspis_check, aspis_detect, aspis_select, aspis_aggregate) is timed after
+it, pass by pass (keys "passes_ms", "roofline_check", "roofline_aggregate").
 
 Default workload: K=15 workers, r=3, f=455 files, d=11,173,962 fp32 (a
 flattened ResNet-18 gradient), optimal (strong) attack with q=3 colluding
@@ -270,9 +272,10 @@ def hbm_entry(kernel, nbytes, ms, peak, peak_kind, traffic=None):
 
 def time_rounds(ap, torch, w, a, copies, buf, stream, steps, warmup, mode, flush=None,
                 clock_gpu=None, dist=None):
-    """Times `steps` rounds (check, detect, select, aggregate) on `stream`
-    with events around every step and every pass.  Returns the per-step pass
-    times, the total (max over ranks when `dist` is set) and the clocks."""
+    """Times `steps` rounds (aspis_round) on `stream` with events around every
+    step, then the separate passes over the same copies.  Returns the total (max
+    over ranks when `dist` is set), the clocks, the passes' times and the kernels
+    of one round."""
     from paper_2108_02416_gb300.shard import max_over_ranks
 
     def one_round(ev=None):
@@ -280,16 +283,22 @@ def time_rounds(ap, torch, w, a, copies, buf, stream, steps, warmup, mode, flush
             flush.zero_()
         if ev:
             ev[0].record(stream)
-        ap.aspis_check(copies, w.d, a, buf.file_neq, buf.adj, stream)
+        ap.aspis_round(copies, w.d, a, buf.file_neq, buf.adj, buf.det, buf.sel, buf.out, mode,
+                       stream)
         if ev:
             ev[1].record(stream)
+
+    def passes(ev):
+        if flush is not None:
+            flush.zero_()
+        ev[0].record(stream)
+        ap.aspis_check(copies, w.d, a, buf.file_neq, buf.adj, stream)
+        ev[1].record(stream)
         ap.aspis_detect(buf.adj, w.K, buf.det, stream)
         ap.aspis_select(buf.file_neq, buf.det, a, buf.sel, stream)
-        if ev:
-            ev[2].record(stream)
+        ev[2].record(stream)
         ap.aspis_aggregate(copies, w.d, a, buf.sel, buf.det, buf.out, mode, stream)
-        if ev:
-            ev[3].record(stream)
+        ev[3].record(stream)
 
     stream.wait_stream(torch.cuda.current_stream())   # inputs were made on the default stream
     with torch.cuda.stream(stream):
@@ -299,7 +308,10 @@ def time_rounds(ap, torch, w, a, copies, buf, stream, steps, warmup, mode, flush
     det = buf.detection()
     if det.status != ap.OK:
         raise RuntimeError(f"{w.name}: round status {ap.status_str(det.status)}")
-    evs = [[torch.cuda.Event(enable_timing=True) for _ in range(4)] for _ in range(steps)]
+    kernels = captured_kernels(torch, stream, one_round)
+    if flush is not None:
+        kernels -= 1              # the flush
+    evs = [[torch.cuda.Event(enable_timing=True) for _ in range(2)] for _ in range(steps)]
     t_start = torch.cuda.Event(enable_timing=True)
     t_end = torch.cuda.Event(enable_timing=True)
     if dist:
@@ -309,10 +321,11 @@ def time_rounds(ap, torch, w, a, copies, buf, stream, steps, warmup, mode, flush
     if clk:
         clk.__enter__()
     try:
-        t_start.record(stream)
-        for k in range(steps):
-            one_round(evs[k])
-        t_end.record(stream)
+        with torch.cuda.stream(stream):
+            t_start.record(stream)
+            for k in range(steps):
+                one_round(evs[k])
+            t_end.record(stream)
         torch.cuda.synchronize()
     finally:
         if clk:
@@ -321,20 +334,64 @@ def time_rounds(ap, torch, w, a, copies, buf, stream, steps, warmup, mode, flush
         dist.barrier()
     total_ms = t_start.elapsed_time(t_end)
     if flush is not None:         # small inputs: exclude the L2 flush kernels
-        total_ms = sum(e[0].elapsed_time(e[3]) for e in evs)
+        total_ms = sum(e[0].elapsed_time(e[1]) for e in evs)
     total_ms = max_over_ranks(total_ms, copies.device)
-    return {"total_ms": total_ms,
-            "check_ms": [e[0].elapsed_time(e[1]) for e in evs],
-            "detsel_ms": [e[1].elapsed_time(e[2]) for e in evs],
-            "agg_ms": [e[2].elapsed_time(e[3]) for e in evs],
-            "det": buf.detection(), "clocks": clk.summary() if clk else None}
+    det, whole = buf.detection(), buf.out.clone()
+    pev = [[torch.cuda.Event(enable_timing=True) for _ in range(4)] for _ in range(steps + 3)]
+    with torch.cuda.stream(stream):
+        for ev in pev:
+            passes(ev)
+    torch.cuda.synchronize()
+    if not torch.equal(whole.view(torch.int32), buf.out.view(torch.int32)):
+        raise RuntimeError(f"{w.name}: aspis_round and the separate calls differ")
+    pev = pev[3:]
+    return {"total_ms": total_ms, "kernels": kernels,
+            "check_ms": [e[0].elapsed_time(e[1]) for e in pev],
+            "detsel_ms": [e[1].elapsed_time(e[2]) for e in pev],
+            "agg_ms": [e[2].elapsed_time(e[3]) for e in pev],
+            "det": det, "clocks": clk.summary() if clk else None}
+
+
+def captured_kernels(torch, stream, call):
+    """Kernels that one call enqueues: the kernel nodes of its capture."""
+    import ctypes
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph, stream=stream):
+        call()
+    cuda = ctypes.CDLL("libcuda.so.1")
+    handle, n, kind = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0), ctypes.c_int(-1)
+    if cuda.cuGraphGetNodes(handle, None, ctypes.byref(n)):
+        raise RuntimeError("cuGraphGetNodes failed")
+    nodes = (ctypes.c_void_p * n.value)()
+    if cuda.cuGraphGetNodes(handle, nodes, ctypes.byref(n)):
+        raise RuntimeError("cuGraphGetNodes failed")
+    kernels = 0
+    for node in nodes:
+        if cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)):
+            raise RuntimeError("cuGraphNodeGetType failed")
+        kernels += kind.value == 0                  # CU_GRAPH_NODE_TYPE_KERNEL
+    return kernels
+
+
+def round_entry(w, n_sel, kernels, ms, peak, peak_kind, traffic=None):
+    """Roofline of the whole round: in one pass every copy is read once and d
+    coordinates are written; else the chosen copies are read again."""
+    cmp_bytes, agg_bytes = algorithmic_bytes(w, n_sel)
+    one_pass = kernels >= 6        # sample, decide, sweep, decide, repair, (open coordinates)
+    if not one_pass:
+        return hbm_entry("aspis_round (compare, decide, aggregate)", cmp_bytes + agg_bytes, ms,
+                         peak, peak_kind)
+    return hbm_entry(f"aspis_round in one pass (sweep_kernel<{w.r}>)", cmp_bytes + w.d * 4, ms,
+                     peak, peak_kind, traffic)
 
 
 def config_entry(w, t, steps, peak, peak_kind):
     n_sel = t["det"].n_sel
     cmp_bytes, agg_bytes = algorithmic_bytes(w, n_sel)
     det = t["det"]
-    return {"round_ms": t["total_ms"] / steps,
+    ms = t["total_ms"] / steps
+    return {"round_ms": ms, "kernels_per_round": t["kernels"],
+            "round": round_entry(w, n_sel, t["kernels"], ms, peak, peak_kind),
             "compare": hbm_entry("compare (aspis_check)", cmp_bytes, statistics.mean(t["check_ms"]),
                                  peak, peak_kind),
             "median": hbm_entry("aggregate (lower median)", agg_bytes,
@@ -555,12 +612,17 @@ def main():
     cmp_bytes, agg_bytes = algorithmic_bytes(w, n_sel)
     peak, peak_kind = peaks()
     ms_round = total_ms / args.steps            # per replica (the slowest one)
-    all_gbs = (cmp_bytes + agg_bytes) / (ms_round * 1e-3) / 1e9
     csrc = os.path.join(ROOT, "paper_2108_02416_gb300", "csrc")
     cmp_traffic = profile_traffic("compare_vec_kernel", w.name, w.f * w.r * w.d,
                                   os.path.join(csrc, "check.cu"))
-    agg_traffic = profile_traffic("aggregate_kernel", w.name, n_sel * w.d,
-                                  os.path.join(csrc, "aggregate.cu"))
+    sweep_src = os.path.join(csrc, "sweep_impl.cuh")
+    if a.f > 1330:                 # more files than a tile's tag bytes hold
+        agg_traffic = profile_traffic("aggregate_kernel", w.name, n_sel * w.d,
+                                      os.path.join(csrc, "aggregate.cu"))
+    else:
+        agg_traffic = profile_traffic("sweep_kernel<1>", w.name, n_sel * w.d, sweep_src)
+    whole = round_entry(w, n_sel, t["kernels"], ms_round, peak, peak_kind,
+                        profile_traffic(f"sweep_kernel<{w.r}>", w.name, w.f * w.r * w.d, sweep_src))
     main_entry = config_entry(w, t, args.steps, peak, peak_kind)
 
     # ---- the model update on the round's output, timed alone: w, v <- Eq. 1
@@ -738,7 +800,6 @@ def main():
         if dist:
             dist.destroy_process_group()
         return
-    launches_per_round = 5    # compare, graph, detect, select, aggregate
     rounds_per_s = world * args.steps / (total_ms * 1e-3)
     line = {
         "metric": metric_name(w), "value": ms_round, "unit": "ms/round", "n_gpus": world,
@@ -749,9 +810,10 @@ def main():
                              f"replicas x{world}: independent full rounds, no collective"),
         "mode": "single" if world == 1 else "replicas",
         "rounds_per_s": rounds_per_s,
-        "gbps": all_gbs,
-        "roofline": dict(hbm_entry("compare (aspis_check)", cmp_bytes, statistics.mean(check_ms),
-                                   peak, peak_kind, cmp_traffic)),
+        "gbps": whole["achieved"],
+        "roofline": whole,
+        "roofline_check": hbm_entry("compare (aspis_check)", cmp_bytes, statistics.mean(check_ms),
+                                    peak, peak_kind, cmp_traffic),
         "roofline_aggregate": hbm_entry("aggregate (lower median)", agg_bytes,
                                         statistics.mean(agg_ms), peak, peak_kind, agg_traffic),
         "passes_ms": {"check": statistics.mean(check_ms),
@@ -760,7 +822,7 @@ def main():
         "detection": {"omega": det.omega, "n_max_cliques": det.n_max_cliques,
                       "success": det.success, "n_sel": n_sel},
         "clocks": clocks,
-        "gpu_launches": launches_per_round * args.steps,
+        "gpu_launches": t["kernels"] * args.steps,
         "e2e": e2e,
         "cpu_baseline": cpu,
         "update": update,
