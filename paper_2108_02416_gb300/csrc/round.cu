@@ -401,16 +401,28 @@ cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, in
 // resident block at a time, and a last wave that is nearly empty costs about
 // 0.4 of a full one (its blocks have the bandwidth for themselves): the one-pass
 // mean of 3,003 files of five copies takes 550 us against 482 with 316 tiles
-// on 304 blocks, 1,309 against 1,355 with 1,024.
-bool one_pass_pays(int64_t f, int r, int64_t d, int mode)
+// on 304 blocks, 1,309 against 1,355 with 1,024.  pairs: rows 8-byte aligned.
+bool one_pass_pays(int64_t f, int r, int64_t d, int mode, bool pairs)
 {
     // few files (35 of three, d = 11,173,962): 1,223 us apart, 1,332 with the copies
     // compared and sorted in registers in one pass, 1,736 with the tile kernel
     if (mode == 0 && f <= kFewFiles) return false;
     const bool many = mode == 0 && f > kTagFiles;                       // two passes over the chosen rows
-    if (f * r * d < (many ? 10 : 1) * kMinValues) return false;
     const int64_t tiles = (d + 127) / 128;
     const int64_t blocks = (int64_t)sm_count() * (mode == 1 || many || f <= kPairFiles ? 2 : 1);
+    if (many && f * r * d < 10 * kMinValues) {
+        // Few tiles: by how full the last wave is (3,003 files of five on 304
+        // blocks, one pass and apart in us: 125 tiles 423 and 449, 256 tiles
+        // 514 and 744, 304 tiles 600 and 670, 352 tiles 923 and 686, 469 tiles
+        // 984 and 1,034; 4,368 files, 256 tiles: 782 and 965).  Up to about 2,700
+        // files the separate median has tags and one pass of its own (2,002
+        // files, 256 tiles: 389 and 306).  Fewer copies leave too little to save (2,024 files
+        // of three, 304 tiles: 307 and 255; 5,985 of four 1,801 and 1,655), and
+        // so do rows of 4-byte loads (257 tiles: 609 and 537).
+        const int64_t last = tiles % blocks;
+        return r == 5 && f > 2700 && pairs && f * r * d >= 2 * kMinValues && (last == 0 || last * 5 >= blocks * 2);
+    }
+    if (f * r * d < kMinValues) return false;
     const double full = (double)((tiles + blocks - 1) / blocks * blocks) / (double)tiles;
     const double wave = 1.0 + 0.4 * (full - 1.0);
     const double all = (double)f * r * (double)d * 4e-6, chosen = all / r;      // MB: us at 1 TB/s
@@ -439,7 +451,7 @@ cudaError_t launch_round_fused(bool &done, const float *copies, int64_t f, int r
                                int8_t *sel, int mode, float *out, cudaStream_t stream)
 {
     done = false;
-    if (r > 5 || !one_pass_pays(f, r, d, mode)) return cudaSuccess;
+    if (r > 5 || !one_pass_pays(f, r, d, mode, (uintptr_t)copies % 8 == 0 && ld % 2 == 0)) return cudaSuccess;
     const SweepArgs A{copies, d, ld, (int)f, sel, det, out, file_neq, r, nullptr, nullptr, nullptr, 0};
     switch (r) {
     case 2: return fused<2>(done, A, fw, K, adj, sel, mode, stream);
