@@ -28,6 +28,7 @@
 #include "aspis_internal.cuh"
 #include "detect_common.cuh"
 #include "median_common.cuh"
+#include "settle.cuh"
 #include "sweep.cuh"
 
 namespace aspis {
@@ -154,171 +155,87 @@ decide_kernel(uint32_t *__restrict__ file_neq, const uint8_t *__restrict__ fw, i
 // The coordinates that the sweep left open (kOpen in out): a NaN among the
 // values, a value bin with more members than a list holds, an overflowed
 // counter, no spread in the sample.  Returns at once when det says that there
-// are none.  A block takes 32 coordinates at a time.
-//   Few of them open: one after the other, the values spread over the block's
-//   threads and their keys selected bit by bit (a load latency and 32 block
-//   counts).
-//   Else an 8-bit radix select of all 32 at once: four passes over the rows'
-//   128-byte segments, which stay in L2.
-constexpr int kFixThreads = 512, kFixWarps = kFixThreads / 32;
-constexpr int kFixPer = ASPIS_MAX_AGG_FILES / kFixThreads;
-constexpr int kFixFew = 6;
-static_assert(kFixPer * kFixThreads == ASPIS_MAX_AGG_FILES, "every kept value has a thread");
+// are none.  A block looks through 32 * masks coordinates at a time (32 at a time
+// took 50 us for a few open ones among 1,048,576) and settles what it finds, up
+// to `most` of 32 neighbours together.
+constexpr int kFixThreads = 256, kFixWarps = kFixThreads / 32, kFixMasks = 32;
+
+__host__ __device__ constexpr size_t fixup_rows(int f)
+{
+    return ((size_t)f * 2 + 15) / 16 * 16;
+}
 
 __global__ void __launch_bounds__(kFixThreads)
-fixup_kernel(const SweepArgs A)
+fixup_kernel(const SweepArgs A, int masks, int most)
 {
     chain();
     if (*(volatile const uint32_t *)&A.det->median_exact == 0u) return;
     extern __shared__ __align__(16) unsigned char smem[];
-    uint32_t *hist = reinterpret_cast<uint32_t *>(smem);              // [256][32]
-    uint16_t *rows = reinterpret_cast<uint16_t *>(hist + 256 * 32);   // kept rows
+    uint16_t *rows = reinterpret_cast<uint16_t *>(smem);              // kept rows
+    uint32_t *stage = reinterpret_cast<uint32_t *>(smem + fixup_rows(A.f));
     __shared__ int warp_tot[kFixWarps];
-    __shared__ uint32_t pre[32], rnk[32], open_s;
-    __shared__ __align__(16) int counts[2][kFixWarps];
+    __shared__ uint32_t open_s[kFixMasks];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, f = A.f;
     const unsigned full = 0xffffffffu;
-    const uint32_t *copies = reinterpret_cast<const uint32_t *>(A.copies);
-    const int64_t ntiles = (A.d + 31) / 32;
+    const int64_t step = (int64_t)gridDim.x * 32;
     int n = -1;
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const int64_t c0 = t * 32;
-        if (w == 0) {
-            const uint32_t x = c0 + lane < A.d ? __float_as_uint(A.out[c0 + lane]) : 0u;
+    for (int64_t c0 = (int64_t)blockIdx.x * 32; c0 < A.d; c0 += masks * step) {
+        uint32_t any = 0u;
+        for (int g = w; g < masks; g += kFixWarps) {
+            const int64_t c = c0 + g * step + lane;
+            const uint32_t x = c < A.d ? __float_as_uint(A.out[c]) : 0u;
             const uint32_t m = __ballot_sync(full, x == kOpen);
-            if (lane == 0) open_s = m;
+            if (lane == 0) open_s[g] = m;
+            any |= m;
         }
-        __syncthreads();
-        uint32_t open = open_s;
-        __syncthreads();
-        if (!open) continue;
-        if (n < 0) {                       // the kept rows, once a block has work
+        if (!__syncthreads_or(any != 0u)) continue;
+        if (n < 0) {                       // the kept rows, once a block has work: a part of the files per warp
+            const int per = (f + kFixThreads - 1) / kFixThreads * 32, i0 = w * per, i1 = min(f, i0 + per);
+            int mine = 0;
+#pragma unroll 4
+            for (int i = i0 + lane; i < i0 + per; i += 32) mine += i < i1 && A.sel[i] >= 0;
+            mine = __reduce_add_sync(full, mine);
+            if (lane == 0) warp_tot[w] = mine;
+            __syncthreads();
+            int off = 0;
             n = 0;
-            for (int b0 = 0; b0 < f; b0 += kFixThreads) {
-                const int i = b0 + tid, s = i < f ? (int)A.sel[i] : -1;
+            for (int q = 0; q < kFixWarps; ++q) {
+                off += q < w ? warp_tot[q] : 0;
+                n += warp_tot[q];
+            }
+            for (int i = i0 + lane; i < i0 + per; i += 32) {
+                const int s = i < i1 ? (int)A.sel[i] : -1;
                 const unsigned m = __ballot_sync(full, s >= 0);
-                if (lane == 0) warp_tot[w] = __popc(m);
-                __syncthreads();
-                int off = n;
-                for (int q = 0; q < kFixWarps; ++q) {
-                    off += q < w ? warp_tot[q] : 0;
-                    n += warp_tot[q];
-                }
                 if (s >= 0) rows[off + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(i * A.r + s);
-                __syncthreads();
-            }
-        }
-        const uint32_t krank = (uint32_t)((n - 1) / 2);
-        if (__popc(open) <= kFixFew) {
-            for (; open; open &= open - 1u) {
-                const int64_t c = c0 + __ffs(open) - 1;
-                uint32_t key[kFixPer];
-#pragma unroll
-                for (int u = 0; u < kFixPer; ++u) {
-                    const int i = tid + u * kFixThreads;
-                    key[u] = i < n ? to_key(__ldcg(copies + (int64_t)rows[i] * A.ld + c)) : 0u;
-                }
-                uint32_t prefix = 0u, rk = krank;
-                for (int b = 31; b >= 0; --b) {
-                    // keys that match the prefix above bit b and have bit b clear
-                    int below = 0;
-#pragma unroll
-                    for (int u = 0; u < kFixPer; ++u)
-                        below += tid + u * kFixThreads < n && (key[u] >> b) == (prefix >> b);
-                    below = __reduce_add_sync(full, below);
-                    if (lane == 0) counts[b & 1][w] = below;
-                    __syncthreads();
-                    below = 0;
-#pragma unroll
-                    for (int q = 0; q < kFixWarps; ++q) below += counts[b & 1][q];
-                    if (rk >= (uint32_t)below) {
-                        rk -= (uint32_t)below;
-                        prefix |= 1u << b;
-                    }
-                }
-                __syncthreads();
-                if (tid == 0) A.out[c] = __uint_as_float(from_key(prefix));
+                off += __popc(m);
             }
             __syncthreads();
-            continue;
+            if (n == 0) return;            // (these were the caller's own bits)
         }
-        const bool live = c0 + lane < A.d;
-        if (tid < 32) {
-            pre[tid] = 0u;
-            rnk[tid] = krank;
-        }
-        for (int p = 0; p < 4; ++p) {
-            const int sh = 24 - 8 * p;
-            const uint32_t pmask = p == 0 ? 0u : 0xFFFFFFFFu << (32 - 8 * p);
-            for (int i = tid; i < 256 * 32; i += kFixThreads) hist[i] = 0u;
-            __syncthreads();
-            const uint32_t want = pre[lane];
-            for (int j0 = w; j0 < n; j0 += kFixWarps * 8) {
-                uint32_t v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int j = j0 + u * kFixWarps;
-                    v[u] = live && j < n ? __ldcg(copies + (int64_t)rows[j] * A.ld + c0 + lane) : 0u;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int j = j0 + u * kFixWarps;
-                    const uint32_t key = to_key(v[u]);
-                    if (live && j < n && (key & pmask) == want) atomicAdd(&hist[((key >> sh) & 0xFFu) * 32 + lane], 1u);
-                }
+        for (int g = 0; g < masks; ++g)
+            for (uint32_t left = open_s[g], open; left; left &= ~open) {
+                open = __popc(left) <= most ? left : left & ((2u << __fns(left, 0, most)) - 1u);
+                settle<kFixThreads>(A.copies, A.ld, n, [&](int i) { return rows[i]; }, c0 + g * step, open, stage,
+                                    A.out);
             }
-            __syncthreads();
-            // a warp settles two coordinates: a warp scan over the 256 digits
-            for (int cc = w; cc < 32; cc += kFixWarps) {
-                uint32_t cb[8], sum = 0u;
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    cb[b] = hist[(lane * 8 + b) * 32 + cc];
-                    sum += cb[b];
-                }
-                uint32_t inc = sum;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t y = __shfl_up_sync(full, inc, o);
-                    if (lane >= o) inc += y;
-                }
-                const uint32_t rk = rnk[cc], exc = inc - sum;
-                const bool mine = exc <= rk && rk < inc;
-                uint32_t dig = 0u, r2 = rk - exc;
-                if (mine) {
-                    bool hit = false;
-#pragma unroll
-                    for (int b = 0; b < 8; ++b) {
-                        if (!hit && r2 < cb[b]) {
-                            dig = (uint32_t)(lane * 8 + b);
-                            hit = true;
-                        }
-                        if (!hit) r2 -= cb[b];
-                    }
-                }
-                const unsigned bal = __ballot_sync(full, mine);
-                const int src = bal ? __ffs(bal) - 1 : 0;
-                dig = __shfl_sync(full, dig, src);
-                r2 = __shfl_sync(full, r2, src);
-                if (lane == 0 && bal) {
-                    pre[cc] |= dig << sh;
-                    rnk[cc] = r2;
-                }
-            }
-            __syncthreads();
-        }
-        if (w == 0 && ((open >> lane) & 1u)) A.out[c0 + lane] = __uint_as_float(from_key(pre[lane]));
         __syncthreads();
     }
 }
 
+// Keys of 32 neighbours where three blocks share an SM, of 16 where two do,
+// else of 8 (a sector of every row).
 cudaError_t launch_fixup(const SweepArgs &A, cudaStream_t stream)
 {
-    const size_t smem = 256 * 32 * 4 + ((size_t)A.f * 2 + 15) / 16 * 16;
-    const int64_t ntiles = (A.d + 31) / 32;
-    int64_t grid = (int64_t)sm_count() * 4;
-    if (grid > ntiles) grid = ntiles;
-    return launch_chained(fixup_kernel, grid, kFixThreads, smem, stream, A);
+    const int most = A.f <= 544 ? 32 : A.f <= 1632 ? 16 : 8;
+    const size_t smem = fixup_rows(A.f) + (size_t)settle_words(A.f, most) * 4;
+    static Residency resident;
+    const int per_sm = resident.blocks(fixup_kernel, kFixThreads, smem);
+    if (per_sm < 1) return cudaErrorInvalidValue;
+    const int64_t masks = (A.d + 31) / 32;
+    int64_t grid = (int64_t)sm_count() * per_sm;
+    if (grid > masks) grid = masks;
+    const int64_t at_once = (masks + grid - 1) / grid < kFixMasks ? (masks + grid - 1) / grid : kFixMasks;
+    return launch_chained(fixup_kernel, grid, kFixThreads, smem, stream, A, (int)at_once, most);
 }
 
 template <int R>

@@ -2,6 +2,7 @@
 // sweep_r*.cu.
 #pragma once
 
+#include "settle.cuh"
 #include "sweep.cuh"
 
 namespace aspis {
@@ -28,9 +29,13 @@ constexpr int TC = 128;                     // coordinates per tile, four per la
 // without tags, from a second pass over the chosen rows.
 enum Mode { TAGGED = 0, MEAN = 1, TWO_PASS = 2 };
 // List entries per coordinate (CAP; the two-pass median's bins are wider).  A
-// bin has n / 120 members on average; half the list lets two blocks share the
-// SM up to kPairFiles files (456 with 32 entries), and 16 are hardly ever
-// exceeded there.
+// bin has n / 120 members on average.  Two blocks share the SM up to 456 files
+// with 32 entries and up to kPairFiles with 16, which are hardly ever exceeded
+// there by continuous values; values kept in 16 bits, whose grid is coarser than
+// the bins, do exceed them (495 files, d = 524,288: 251 us, 647 with gradients of
+// bf16; with a block alone 390 and 440).  A block alone takes 64 where they fit
+// (kLongFiles): of such values at 816 files it leaves 881 coordinates of 524,288
+// open, not 56,173 (672 us, not 1,136).
 template <int MODE, int CAP>
 __host__ __device__ constexpr int list_cap() { return MODE == TWO_PASS ? 96 : CAP; }
 constexpr int kHistWords = kVB * 32;        // four 8-bit counters per (bin, lane)
@@ -176,139 +181,26 @@ __device__ __forceinline__ int warp_ranked(uint32_t a, uint32_t b, uint32_t cnt,
 
 // The coordinates that a block left open (kOpen in its part of out), at the end
 // of its sweep, where there are so few tiles that fixup_kernel's launch would
-// cost more (27 -> 24 us at 35 files of three, d = 4,096).  In larger calls the
-// mere presence of this call costs the sweep 5 to 9%.  32 coordinates at a time.
-//   Few of them open: one after the other, the values spread over the block's
-//   threads and their keys selected bit by bit (a load latency and 32 block
-//   counts: 5 to 10 us).
-//   Else an 8-bit radix select of all 32 at once: four passes over the rows'
-//   128-byte segments.
-__device__ __noinline__ void settle_open(const SweepArgs &A, uint32_t *hist, const uint32_t *meta, int n,
+// cost more.  In larger calls the mere presence of this call costs the sweep 5
+// to 9%.  stage: room for 32 coordinates' keys.
+__device__ __noinline__ void settle_open(const SweepArgs &A, uint32_t *stage, const uint32_t *meta, int n,
                                          int64_t t0, int64_t tstep)
 {
-    constexpr int kPer = (ASPIS_MAX_AGG_FILES + kNT - 1) / kNT, kFew = 6;
-    __shared__ uint32_t pre[32], rnk[32], open_s;
-    __shared__ int counts[2][kWarps];
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const unsigned full = 0xffffffffu;
-    const uint32_t krank = (uint32_t)((n - 1) / 2);
-    // the i-th kept row, NULL: none
-    auto row_of = [&](int i) -> const uint32_t * {
-        return i < n ? reinterpret_cast<const uint32_t *>(A.copies) + (int64_t)meta[i] * A.ld : nullptr;
-    };
-    const int64_t groups = (A.d + 31) / 32;
-    for (int64_t g0 = t0 * (TC / 32); g0 < groups; g0 += tstep * (TC / 32))
-        for (int64_t g = g0; g < g0 + TC / 32 && g < groups; ++g) {
-            const int64_t c0 = g * 32;
-            if (w == 0) {
-                const uint32_t x = c0 + lane < A.d ? __ldcg(reinterpret_cast<const unsigned int *>(A.out) + c0 + lane) : 0u;
-                const uint32_t m = __ballot_sync(full, x == kOpen);
-                if (lane == 0) open_s = m;
-            }
-            __syncthreads();
-            uint32_t open = open_s;
-            __syncthreads();
-            if (!open) continue;
-            if (__popc(open) <= kFew) {
-                for (; open; open &= open - 1u) {
-                    const int64_t c = c0 + __ffs(open) - 1;
-                    uint32_t key[kPer], has = 0u;
-#pragma unroll
-                    for (int u = 0; u < kPer; ++u) {
-                        const uint32_t *row = row_of(tid + u * kNT);
-                        key[u] = row ? to_key(__ldcg(row + c)) : 0u;
-                        has |= (row ? 1u : 0u) << u;
-                    }
-                    uint32_t prefix = 0u, rk = krank;
-                    for (int b = 31; b >= 0; --b) {
-                        // keys that match the prefix above bit b and have bit b clear
-                        int below = 0;
-#pragma unroll
-                        for (int u = 0; u < kPer; ++u) below += ((has >> u) & 1u) && (key[u] >> b) == (prefix >> b);
-                        below = __reduce_add_sync(full, below);
-                        if (lane == 0) counts[b & 1][w] = below;
-                        __syncthreads();
-                        below = 0;
-#pragma unroll
-                        for (int q = 0; q < kWarps; ++q) below += counts[b & 1][q];
-                        if (rk >= (uint32_t)below) {
-                            rk -= (uint32_t)below;
-                            prefix |= 1u << b;
-                        }
-                    }
-                    __syncthreads();
-                    if (tid == 0) A.out[c] = __uint_as_float(from_key(prefix));
-                }
-                __syncthreads();
-                continue;
-            }
-            const bool live = c0 + lane < A.d;
-            if (tid < 32) {
-                pre[tid] = 0u;
-                rnk[tid] = krank;
-            }
-            for (int p = 0; p < 4; ++p) {
-                const int sh = 24 - 8 * p;
-                const uint32_t pmask = p == 0 ? 0u : 0xFFFFFFFFu << (32 - 8 * p);
-                for (int i = tid; i < 256 * 32; i += kNT) hist[i] = 0u;
-                __syncthreads();
-                const uint32_t want = pre[lane];
-                for (int j0 = w; j0 < n; j0 += kWarps * 8) {
-                    uint32_t v[8], has = 0u;
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const uint32_t *row = live ? row_of(j0 + u * kWarps) : nullptr;
-                        v[u] = row ? __ldcg(row + c0 + lane) : 0u;
-                        has |= (row ? 1u : 0u) << u;
-                    }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const uint32_t key = to_key(v[u]);
-                        if (((has >> u) & 1u) && (key & pmask) == want)
-                            atomicAdd(&hist[((key >> sh) & 0xFFu) * 32 + lane], 1u);
-                    }
-                }
-                __syncthreads();
-                // a warp settles a digit of a coordinate: a warp scan over the 256 counts
-                for (int cc = w; cc < 32; cc += kWarps) {
-                    uint32_t cb[8], sum = 0u;
-#pragma unroll
-                    for (int b = 0; b < 8; ++b) {
-                        cb[b] = hist[(lane * 8 + b) * 32 + cc];
-                        sum += cb[b];
-                    }
-                    uint32_t inc = sum;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const uint32_t y = __shfl_up_sync(full, inc, o);
-                        if (lane >= o) inc += y;
-                    }
-                    const uint32_t rk = rnk[cc], exc = inc - sum;
-                    const bool mine = exc <= rk && rk < inc;
-                    uint32_t dig = 0u, r2 = rk - exc;
-                    bool hit = false;
-#pragma unroll
-                    for (int b = 0; b < 8; ++b) {
-                        if (!hit && r2 < cb[b]) {
-                            dig = (uint32_t)(lane * 8 + b);
-                            hit = true;
-                        }
-                        if (!hit) r2 -= cb[b];
-                    }
-                    const unsigned bal = __ballot_sync(full, mine);
-                    const int src = bal ? __ffs(bal) - 1 : 0;
-                    dig = __shfl_sync(full, dig, src);
-                    r2 = __shfl_sync(full, r2, src);
-                    if (lane == 0 && bal) {
-                        pre[cc] |= dig << sh;
-                        rnk[cc] = r2;
-                    }
-                }
-                __syncthreads();
-            }
-            if (w == 0 && ((open >> lane) & 1u)) A.out[c0 + lane] = __uint_as_float(from_key(pre[lane]));
-            __syncthreads();
+    __shared__ uint32_t open_s[TC / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int64_t c0 = t0 * TC; c0 < A.d; c0 += tstep * TC) {
+        if (w < TC / 32) {
+            const int64_t c = c0 + w * 32 + lane;
+            const uint32_t x = c < A.d ? __ldcg(reinterpret_cast<const unsigned int *>(A.out) + c) : 0u;
+            const uint32_t m = __ballot_sync(0xffffffffu, x == kOpen);
+            if (lane == 0) open_s[w] = m;
         }
+        __syncthreads();
+        for (int g = 0; g < TC / 32; ++g)
+            if (open_s[g])
+                settle<kNT>(A.copies, A.ld, n, [&](int i) { return meta[i]; }, c0 + g * 32, open_s[g], stage, A.out);
+        __syncthreads();
+    }
 }
 
 // AVG: a file's value is the average of its copies in slot_mask; the meta word
@@ -504,13 +396,13 @@ sweep_kernel(const SweepArgs A)
         for (int q = (w - TC / 32 + kWarps) % kWarps; q < nl; q += kWarps) {
             const int c = long_c[q];
             const uint32_t cnt = S(S_PEND, c) & 0xFFu, rk = S(S_PEND, c) >> 8;
-            if (MODE == TAGGED || cnt <= 32u) {
+            if (cap <= 32u || cnt <= 32u) {
                 const uint32_t x = warp_sort32((uint32_t)lane < cnt ? to_key(list[lane * TC + c]) : 0xffffffffu, lane);
                 const uint32_t res = __shfl_sync(full, x, (int)rk);
                 if (lane == 0) A.out[c0_p + seg_at<W>(c)] = __uint_as_float(from_key(res));
                 continue;
             }
-            if (cnt <= 64u) {
+            if (cap <= 64u || cnt <= 64u) {
                 // (equal keys: several lanes write the same bits)
                 const uint32_t a = list[lane * TC + c], b = (uint32_t)lane + 32u < cnt ? list[(lane + 32) * TC + c] : 0u;
                 const int is = warp_ranked(to_key(a), to_key(b), cnt, rk);
@@ -932,7 +824,9 @@ sweep_kernel(const SweepArgs A)
             if (lane == 0 && open_cnt) atomicAdd(&A.det->median_exact, open_cnt);
         }
         if constexpr (SETTLE) {
-            if (__syncthreads_or(open_cnt != 0u)) settle_open(A, hist, meta, n, blockIdx.x, gridDim.x);
+            // (the tags and the counters after them are done with)
+            static_assert(kHistWords >= 32 * 32, "the tags' f rows of 32 words are up to 32 rows short of the keys");
+            if (__syncthreads_or(open_cnt != 0u)) settle_open(A, tags, meta, n, blockIdx.x, gridDim.x);
         }
     }
     if constexpr (R == 1) {
@@ -977,7 +871,8 @@ cudaError_t sweep_for(bool &ok, bool &open, const SweepArgs &A, int mode, bool c
     cudaError_t e = cudaSuccess;
     if constexpr (R == 1) {
         if (alone && A.f <= kTagFiles) {
-            e = try_sweep<R, W, TAGGED, 1, false, 32, true>(ok, A, chained, stream);
+            e = A.f <= kLongFiles ? try_sweep<R, W, TAGGED, 1, false, 64, true>(ok, A, chained, stream)
+                                  : try_sweep<R, W, TAGGED, 1, false, 32, true>(ok, A, chained, stream);
             if (ok) open = false;
             return e;
         }
@@ -987,7 +882,9 @@ cudaError_t sweep_for(bool &ok, bool &open, const SweepArgs &A, int mode, bool c
             e = try_sweep<R, W, TAGGED, 2>(ok, A, chained, stream);
             if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 2, false, 16>(ok, A, chained, stream);
         }
-        if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 1>(ok, A, chained, stream);
+        if (e == cudaSuccess && !ok)
+            e = A.f <= kLongFiles ? try_sweep<R, W, TAGGED, 1, false, 64>(ok, A, chained, stream)
+                                  : try_sweep<R, W, TAGGED, 1>(ok, A, chained, stream);
         if (e != cudaSuccess || ok) return e;
     }
     return try_sweep<R, W, TWO_PASS, 2>(ok, A, chained, stream);
@@ -1011,7 +908,9 @@ cudaError_t launch_sweep_averages(bool &ok, const SweepArgs &A, cudaStream_t str
     const bool chained = false;
     cudaError_t e = cudaSuccess;
     if ((A.d + TC - 1) / TC > sm_count()) e = try_sweep<R, 4, TAGGED, 2, true>(ok, A, chained, stream);
-    if (e == cudaSuccess && !ok) e = try_sweep<R, 4, TAGGED, 1, true>(ok, A, chained, stream);
+    if (e == cudaSuccess && !ok)
+        e = A.f <= kLongFiles ? try_sweep<R, 4, TAGGED, 1, true, 64>(ok, A, chained, stream)
+                              : try_sweep<R, 4, TAGGED, 1, true>(ok, A, chained, stream);
     return e;
 }
 
