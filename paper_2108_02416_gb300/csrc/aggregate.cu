@@ -48,6 +48,7 @@
 
 #include "aspis_internal.cuh"
 #include "median_common.cuh"
+#include "sweep.cuh"
 
 namespace aspis {
 namespace {
@@ -121,7 +122,9 @@ __host__ __device__ inline Layout make_layout(int64_t f)
     return L;
 }
 
-template <int V, int MINB, bool W32, int MODE, int NT>
+// LEAVE: coordinates that need the exact passes are left open for fixup_kernel
+// (round.cu).
+template <int V, int MINB, bool W32, int MODE, int NT, bool LEAVE>
 __global__ void __launch_bounds__(NT, MINB)
 aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, int64_t ld,
                  const int8_t *__restrict__ sel, aspis_detection *det, float *__restrict__ out)
@@ -222,7 +225,7 @@ aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, 
     }
     __syncthreads();
 
-    uint32_t exact_cnt = 0u;        // coordinates resolved by the exact passes (thread 0)
+    uint32_t exact_cnt = 0u;        // coordinates resolved by the exact passes (thread 0), or left open
 
     // The previous tile ("pending"): its median bins are known, its members
     // are listed during the next sweep and ranked after it.
@@ -550,11 +553,19 @@ aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, 
                 S(S_PCNT, c) = pc;
                 if (pc > (uint32_t)kShort) long_c[atomicAdd(&n_long, 1)] = (uint8_t)c;
                 const uint32_t mdn = S(S_MODE, c);
-                if (mdn == M_VM || mdn == M_KA) any_exact = 1;
+                if (mdn == M_VM || mdn == M_KA) {
+                    if constexpr (LEAVE) {
+                        S(S_MODE, c) = M_DONE;
+                        out[c0 + c] = __uint_as_float(kOpen);
+                        ++exact_cnt;
+                    } else {
+                        any_exact = 1;
+                    }
+                }
             }
             __syncthreads();                                        // (E)
             // the same in every thread: no barrier decides the exact passes
-            const bool exact_pass = any_exact != 0;
+            const bool exact_pass = !LEAVE && any_exact != 0;
             for (int i = tid * 4; i < HW; i += kThreads * 4)
                 *reinterpret_cast<uint4 *>(hist + i) = make_uint4(0u, 0u, 0u, 0u);
 
@@ -803,7 +814,7 @@ aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, 
             __syncthreads();
             rank_pending();
         }
-        if (tid == 0 && exact_cnt) atomicAdd(&det->median_exact, exact_cnt);
+        if (exact_cnt) atomicAdd(&det->median_exact, exact_cnt);
     }
 }
 
@@ -934,7 +945,7 @@ median_radix_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t 
     }
 }
 
-template <int V, int MINB, bool W32, int MODE, int NT>
+template <int V, int MINB, bool W32, int MODE, int NT, bool LEAVE = false>
 cudaError_t try_launch(bool &launched, const float *copies, int64_t f, int r, int64_t d,
                        int64_t ld, const int8_t *sel, aspis_detection *det, float *out,
                        cudaStream_t stream)
@@ -942,7 +953,7 @@ cudaError_t try_launch(bool &launched, const float *copies, int64_t f, int r, in
     launched = false;
     const Layout L = make_layout<V, NT, MODE>(f);
     if (L.total > smem_cap()) return cudaSuccess;
-    auto kern = aggregate_kernel<V, MINB, W32, MODE, NT>;
+    auto kern = aggregate_kernel<V, MINB, W32, MODE, NT, LEAVE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)L.total);
     if (e != cudaSuccess) return e;
@@ -1003,12 +1014,35 @@ cudaError_t launch_many(int align, const float *copies, int64_t f, int r, int64_
 
 }  // namespace
 
+namespace {
+
+template <bool W32>
+cudaError_t narrow(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld, const int8_t *sel,
+                   aspis_detection *det, float *out, bool few, cudaStream_t stream)
+{
+    const int width = load_width(copies, ld);
+    cudaError_t e = cudaSuccess;
+    if (width >= 2) e = try_launch<2, 2, W32, 0, 384, true>(done, copies, f, r, d, ld, sel, det, out, stream);
+    if (e != cudaSuccess || done || !few || width == 4) return e;
+    return width == 2 ? try_launch<2, 1, W32, 0, 384, true>(done, copies, f, r, d, ld, sel, det, out, stream)
+                      : try_launch<1, 2, W32, 0, 384, true>(done, copies, f, r, d, ld, sel, det, out, stream);
+}
+
+}  // namespace
+
+cudaError_t launch_aggregate_narrow(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
+                                    const int8_t *sel, aspis_detection *det, float *out, bool few,
+                                    cudaStream_t stream)
+{
+    done = false;
+    return (uint64_t)ld * 4u < (1ull << 32) ? narrow<true>(done, copies, f, r, d, ld, sel, det, out, few, stream)
+                                            : narrow<false>(done, copies, f, r, d, ld, sel, det, out, few, stream);
+}
+
 cudaError_t launch_aggregate_many(const float *copies, int64_t f, int r, int64_t d, int64_t ld,
                                   const int8_t *sel, aspis_detection *det, float *out, cudaStream_t stream)
 {
-    // widest load every row start allows: 16 bytes (V = 4), 8 (V = 2), else 4
-    const uintptr_t p = (uintptr_t)copies;
-    const int align = (p % 16 == 0 && ld % 4 == 0) ? 4 : (p % 8 == 0 && ld % 2 == 0) ? 2 : 1;
+    const int align = load_width(copies, ld);              // V = 4, 2 or 1
     const bool w32 = (uint64_t)ld * 4u < (1ull << 32);     // row pitch fits a 32-bit multiplier
     return w32 ? launch_many<true>(align, copies, f, r, d, ld, sel, det, out, stream)
                : launch_many<false>(align, copies, f, r, d, ld, sel, det, out, stream);

@@ -36,6 +36,13 @@ cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, in
 // The lower median for f > kTagFiles (aggregate.cu).
 cudaError_t launch_aggregate_many(const float *copies, int64_t f, int r, int64_t d, int64_t ld,
                                   const int8_t *sel, aspis_detection *det, float *out, cudaStream_t stream);
+// The lower median in 64-coordinate tiles, two blocks per SM where the files'
+// tag bytes allow it; few: else also one block, or (rows of 4-byte alignment)
+// 32-coordinate tiles.  fixup_kernel has to follow.  done = false (and nothing
+// enqueued) where the 128-coordinate tiles of sweep_kernel are better.
+cudaError_t launch_aggregate_narrow(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
+                                    const int8_t *sel, aspis_detection *det, float *out, bool few,
+                                    cudaStream_t stream);
 // At most kFewFiles files (sweep.cuh), median.
 cudaError_t launch_aggregate_few(const float *copies, int64_t f, int r, int64_t d, int64_t ld, const int8_t *sel,
                                  aspis_detection *det, float *out, bool chained, cudaStream_t stream);

@@ -279,6 +279,20 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, i
     // coordinates, against 28 at 2,024 files, d = 9,000) or two passes with
     // more rows in flight (165 against 126 us at 3,003 files).
     if (mode == 0 && f > kTagFiles && !gate) return launch_aggregate_many(copies, f, r, d, ld, sel, det, out, stream);
+    // 517 to 1,330 files: a block of 128-coordinate tiles has an SM to itself.  Up to
+    // about 950 files two of 64-coordinate ones share it (us, wide and narrow, 816
+    // files: 35 and 26 at d = 4,096, 54 and 51 at 36,928, 273 and 243 at 262,144, 988
+    // and 946 at 1,048,576).  Where rows are not 16-byte aligned, narrower tiles are
+    // also better while the wide ones make up to three waves (1,287 files, 4-byte
+    // rows: 60 and 50 at 16,317, 88 and 69 at 24,865, 117 and 108 at 48,173, but 1,560
+    // and 2,640 at 1,048,577).
+    if (mode == 0 && f > kPairFiles && !gate) {
+        bool done = false;
+        const bool few = (d + 127) / 128 <= 3 * (int64_t)sm_count();
+        const cudaError_t e = launch_aggregate_narrow(done, copies, f, r, d, ld, sel, det, out, few, stream);
+        if (e != cudaSuccess) return e;
+        if (done) return launch_fixup(A, stream);
+    }
     bool ok = false, open = false;
     const cudaError_t e = launch_sweep<1>(ok, open, A, mode, chained, stream);
     if (e != cudaSuccess) return e;

@@ -51,6 +51,13 @@ struct SweepArgs {
     int64_t ldm;
 };
 
+// Floats of the widest load that every row start allows.
+inline int load_width(const float *copies, int64_t ld)
+{
+    const uintptr_t p = (uintptr_t)copies;
+    return p % 16 == 0 && ld % 4 == 0 ? 4 : p % 8 == 0 && ld % 2 == 0 ? 2 : 1;
+}
+
 // ok = false where no layout holds f files; open = fixup_kernel has to follow.
 template <int R>
 cudaError_t launch_sweep(bool &ok, bool &open, const SweepArgs &A, int mode, bool chained, cudaStream_t stream);

@@ -895,10 +895,11 @@ cudaError_t sweep_for(bool &ok, bool &open, const SweepArgs &A, int mode, bool c
 template <int R>
 cudaError_t launch_sweep(bool &ok, bool &open, const SweepArgs &A, int mode, bool chained, cudaStream_t stream)
 {
-    const uintptr_t p = (uintptr_t)A.copies;
-    if (p % 16 == 0 && A.ld % 4 == 0) return sweep_for<R, 4>(ok, open, A, mode, chained, stream);
-    if (p % 8 == 0 && A.ld % 2 == 0) return sweep_for<R, 2>(ok, open, A, mode, chained, stream);
-    return sweep_for<R, 1>(ok, open, A, mode, chained, stream);
+    switch (load_width(A.copies, A.ld)) {
+    case 4: return sweep_for<R, 4>(ok, open, A, mode, chained, stream);
+    case 2: return sweep_for<R, 2>(ok, open, A, mode, chained, stream);
+    default: return sweep_for<R, 1>(ok, open, A, mode, chained, stream);
+    }
 }
 
 template <int R>

@@ -38,10 +38,10 @@ def spoil(u, rng):
         u[:, c] = kinds[(k * 5 + k // len(kinds)) % len(kinds)]
 
 
-# the files' number decides how many coordinates are settled together, d whether
+# the files' number and the rows' alignment decide which tiles take them and how many
 # that is done by the tile's own block (one tile per SM) or by the kernel after it
-@pytest.mark.parametrize("K,r", [(8, 3), (15, 3), (12, 4), (16, 3), (18, 3), (20, 3), (21, 3)])
-@pytest.mark.parametrize("d,odd", [(300, 0), (19_600, 0), (19_601, 1)])
+@pytest.mark.parametrize("K,r", [(8, 3), (15, 3), (12, 4), (16, 3), (18, 3), (12, 6), (20, 3), (21, 3)])
+@pytest.mark.parametrize("d,odd", [(300, 0), (19_600, 0), (19_600, 2), (19_601, 1)])
 def test_open_coordinates(K, r, d, odd):
     oa, a = oracle.assign(K, r), ap.aspis_assign(K, r)
     rng = np.random.default_rng(K * d)
