@@ -112,7 +112,7 @@ __host__ __device__ inline Layout make_layout(int64_t f)
     const int64_t per_slot = (f + kWarps - 1) / kWarps;
     const int64_t jw = (per_slot + G::RPW - 1) / G::RPW;     // tag words per thread
     size_t o = 0;
-    // the two-pass median keeps no tags
+    // the mean and the two-pass median keep no tags
     L.tags = o; o += MODE == 0 ? (size_t)jw * kWarps * 32 * 4 : 0;
     L.hist = o; o += (size_t)G::HW * 4;
     L.list = o; o += (size_t)(MODE == 2 ? kListWords2 : kListWords) * 4;   // also the partial sums
@@ -361,7 +361,39 @@ aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, 
             batch(std::true_type{}, j0);
         };
 
-        {
+        if constexpr (MODE == 1) {
+            // ---- mean: compensated per-thread sums, combined in warp order
+            float sm[V], se[V];
+#pragma unroll
+            for (int k = 0; k < V; ++k) sm[k] = se[k] = 0.f;
+            sweep([](int) {}, [&](const T &x, int, int) {
+#pragma unroll
+                for (int k = 0; k < V; ++k) {
+                    float ns, ne;
+                    two_sum(sm[k], __uint_as_float(elem<V>(x, k)), ns, ne);
+                    sm[k] = ns;
+                    se[k] += ne;
+                }
+            }, std::false_type{});
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+                list[(2 * w) * TC + lane * V + k] = __float_as_uint(sm[k]);
+                list[(2 * w + 1) * TC + lane * V + k] = __float_as_uint(se[k]);
+            }
+            __syncthreads();
+            for (int c = tid; c < TC; c += kThreads) {
+                if (c0 + c >= d) continue;
+                float a = 0.f, ae = 0.f;
+                for (int u = 0; u < kWarps; ++u) {
+                    float ns, ne;
+                    two_sum(a, __uint_as_float(list[(2 * u) * TC + c]), ns, ne);
+                    a = ns;
+                    ae += ne + __uint_as_float(list[(2 * u + 1) * TC + c]);
+                }
+                out[c0 + c] = (float)(((double)a + (double)ae) / (double)n);
+            }
+            __syncthreads();
+        } else {
             // ---- S: key range of the sample (rows 0 and 1 of every warp)
             if (lv) {
 #pragma unroll
@@ -807,7 +839,7 @@ aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, 
             }
         }
     }
-    {
+    if constexpr (MODE != 1) {
         // the last tile's listed members are ranked once their copies land
         if (MODE == 0 && have_p) {
             cp_async_wait_all();
@@ -1028,7 +1060,28 @@ cudaError_t narrow(bool &done, const float *copies, int64_t f, int r, int64_t d,
                       : try_launch<1, 2, W32, 0, 384, true>(done, copies, f, r, d, ld, sel, det, out, stream);
 }
 
+template <bool W32>
+cudaError_t mean(const float *copies, int64_t f, int r, int64_t d, int64_t ld, const int8_t *sel,
+                 aspis_detection *det, float *out, cudaStream_t stream)
+{
+    bool ok = false;
+    cudaError_t e;
+    switch (load_width(copies, ld)) {
+    case 4: e = try_launch<4, 2, W32, 1, 384>(ok, copies, f, r, d, ld, sel, det, out, stream); break;
+    case 2: e = try_launch<2, 2, W32, 1, 384>(ok, copies, f, r, d, ld, sel, det, out, stream); break;
+    default: e = try_launch<1, 2, W32, 1, 384>(ok, copies, f, r, d, ld, sel, det, out, stream); break;
+    }
+    return e == cudaSuccess && !ok ? cudaErrorInvalidValue : e;
+}
+
 }  // namespace
+
+cudaError_t launch_aggregate_mean(const float *copies, int64_t f, int r, int64_t d, int64_t ld, const int8_t *sel,
+                                  aspis_detection *det, float *out, cudaStream_t stream)
+{
+    return (uint64_t)ld * 4u < (1ull << 32) ? mean<true>(copies, f, r, d, ld, sel, det, out, stream)
+                                            : mean<false>(copies, f, r, d, ld, sel, det, out, stream);
+}
 
 cudaError_t launch_aggregate_narrow(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
                                     const int8_t *sel, aspis_detection *det, float *out, bool few,

@@ -43,6 +43,9 @@ cudaError_t launch_aggregate_many(const float *copies, int64_t f, int r, int64_t
 cudaError_t launch_aggregate_narrow(bool &done, const float *copies, int64_t f, int r, int64_t d, int64_t ld,
                                     const int8_t *sel, aspis_detection *det, float *out, bool few,
                                     cudaStream_t stream);
+// The mean in tiles of 32 loads of the widest kind that the rows allow.
+cudaError_t launch_aggregate_mean(const float *copies, int64_t f, int r, int64_t d, int64_t ld, const int8_t *sel,
+                                  aspis_detection *det, float *out, cudaStream_t stream);
 // At most kFewFiles files (sweep.cuh), median.
 cudaError_t launch_aggregate_few(const float *copies, int64_t f, int r, int64_t d, int64_t ld, const int8_t *sel,
                                  aspis_detection *det, float *out, bool chained, cudaStream_t stream);

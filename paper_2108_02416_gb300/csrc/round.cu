@@ -293,6 +293,18 @@ cudaError_t launch_aggregate(const float *copies, int64_t f, int r, int64_t d, i
         if (e != cudaSuccess) return e;
         if (done) return launch_fixup(A, stream);
     }
+    // The mean by itself: tiles of 32 loads per row (of 512, 256 or 128 bytes) where
+    // the 128-coordinate tiles are few, and for 8-byte rows of few files (us, wide
+    // and narrow): 455 files, d = 3,661, 23.0 and 17.5; 3,276, 10,172, 62.9 and
+    // 48.0; 1,330, 25,060, 43.9 and 39.3, 250,624, 228 and 224; 4-byte rows of 1,330,
+    // 25,061, 47.2 and 50.0; 8-byte rows of 84, 3,968,254, 410 and 296, of 3,276,
+    // 101,750, 237 and 251.  Within a round the wide tiles start early, which is worth
+    // 3 us (3,003 files of five, d = 6,662: 148 and 126).
+    if (mode == 1 && !gate && (!chained || f > kTagFiles)) {
+        const int width = load_width(copies, ld);
+        if ((d + 127) / 128 <= (width == 1 ? 1 : 4) * (int64_t)sm_count() || (width == 2 && f <= kPairFiles))
+            return launch_aggregate_mean(copies, f, r, d, ld, sel, det, out, stream);
+    }
     bool ok = false, open = false;
     const cudaError_t e = launch_sweep<1>(ok, open, A, mode, chained, stream);
     if (e != cudaSuccess) return e;
