@@ -337,15 +337,14 @@ cudaError_t launch_average_median(bool &done, const float *copies, int64_t f, in
 }
 
 // Whether the one-pass round beats the separate compare and aggregation, from
-// the bytes that each moves and the rates measured for them (TB/s on GB300:
-// compare 7.1, sweep 6.3, the separate median 4.4, mean 5.6, median of more
-// than kTagFiles files 2.7) and the launches (the guess, its check and the
-// empty repair: 30 us against 10).  Tiles of 128 coordinates run one per
-// resident block at a time, and a last wave that is nearly empty costs about
-// 0.4 of a full one (its blocks have the bandwidth for themselves): the one-pass
-// mean of 3,003 files of five copies takes 550 us against 482 with 316 tiles
-// on 304 blocks, 1,309 against 1,355 with 1,024.  pairs: rows 8-byte aligned.
-bool one_pass_pays(int64_t f, int r, int64_t d, int mode, bool pairs)
+// the bytes that each moves, the rates measured for them (TB/s on GB300) and the
+// launches (the guess, its check and the empty repair: 30 us against 10).  Tiles
+// of 128 coordinates run one per resident block at a time, and a last wave that
+// is nearly empty costs about 0.4 of a full one (its blocks have the bandwidth
+// for themselves): the one-pass mean of 3,003 files of five copies takes 550 us
+// against 482 with 316 tiles on 304 blocks, 1,309 against 1,355 with 1,024.
+// width: floats that a row start is aligned to (4, 2 or 1).
+bool one_pass_pays(int64_t f, int r, int64_t d, int mode, int width)
 {
     // few files (35 of three, d = 11,173,962): 1,223 us apart, 1,332 with the copies
     // compared and sorted in registers in one pass, 1,736 with the tile kernel
@@ -353,25 +352,42 @@ bool one_pass_pays(int64_t f, int r, int64_t d, int mode, bool pairs)
     const bool many = mode == 0 && f > kTagFiles;                       // two passes over the chosen rows
     const int64_t tiles = (d + 127) / 128;
     const int64_t blocks = (int64_t)sm_count() * (mode == 1 || many || f <= kPairFiles ? 2 : 1);
-    if (many && f * r * d < 10 * kMinValues) {
-        // Few tiles: by how full the last wave is (3,003 files of five on 304
-        // blocks, one pass and apart in us: 125 tiles 423 and 449, 256 tiles
-        // 514 and 744, 304 tiles 600 and 670, 352 tiles 923 and 686, 469 tiles
-        // 984 and 1,034; 4,368 files, 256 tiles: 782 and 965).  Up to about 2,700
-        // files the separate median has tags and one pass of its own (2,002
-        // files, 256 tiles: 389 and 306).  Fewer copies leave too little to save (2,024 files
-        // of three, 304 tiles: 307 and 255; 5,985 of four 1,801 and 1,655), and
-        // so do rows of 4-byte loads (257 tiles: 609 and 537).
-        const int64_t last = tiles % blocks;
-        return r == 5 && f > 2700 && pairs && f * r * d >= 2 * kMinValues && (last == 0 || last * 5 >= blocks * 2);
+    const double full = (double)((tiles + blocks - 1) / blocks * blocks) / (double)tiles;
+    const double all = (double)f * r * (double)d * 4e-6, chosen = all / r;      // MB: us at 1 TB/s
+    if (many) {
+        // The separate median has tags and one pass in 64-coordinate (rows of 4-byte
+        // alignment: 32-coordinate) tiles up to kNarrowFiles files; beyond them two
+        // passes over 16-byte rows, one in 32-coordinate tiles over others.  Many
+        // rows far apart cost both ways page walks.  Fitted to 15 clusters of 1,540
+        // to 5,985 files, 2 x 10^7 to 6 x 10^9 values and the three alignments; the
+        // better way or one within 5% of it is taken, some of it (one pass and apart
+        // in us):
+        //   16 bytes  1,540 of three   d = 151,512    751 and   817   670,992  2,914 and 3,474
+        //             2,002 of five        104,892  1,007 and   921   309,688  2,586 and 2,677
+        //             2,600 of three       134,612  1,168 and 1,114   397,432  3,021 and 3,165
+        //             3,003 of five         46,620    896 and   880    69,928  1,029 and 1,116
+        //             4,368 of five         32,048    792 and   979    73,260  1,638 and 1,785
+        //    8 bytes  2,002 of five        159,842  1,788 and 1,590   309,690  3,089 and 3,512
+        //             3,276 of three        40,702    716 and   562   162,802  2,009 and 2,231
+        //             4,368 of five         18,314    659 and   486   274,726  6,720 and 6,940
+        //    4 bytes  2,024 of three        32,937    314 and   313   172,925  1,270 and 1,582
+        //             4,845 of four        159,957  4,202 and 3,752   309,597  7,201 and 7,855
+        const double once = (all + chosen) * (1.0 + 0.6 * (full - 1.0));
+        if (f > kNarrowFiles && width < 4)
+            return once / (6.23 - 0.377e-3 * (double)f) + 180.0 < all / 5.7 + chosen / 1.9 + 10.0;
+        if (width == 4)
+            return once / 6.3 + 180.0 <
+                   all / 7.1 + (f <= kNarrowFiles ? chosen / 2.7 + 10.0 : chosen / 2.6 + 0.1 * (double)f - 90.0);
+        return width == 2 ? once / 5.5 + 180.0 < all / 5.8 + chosen / 2.7 + 10.0
+                          : once / 5.4 + 180.0 < all / 5.9 + chosen / 1.75 + 10.0;
     }
     if (f * r * d < kMinValues) return false;
-    const double full = (double)((tiles + blocks - 1) / blocks * blocks) / (double)tiles;
+    // 517 to 1,330 files in 4-byte loads (1,287 of five, d = 48,173: 356 and 330 us;
+    // 1,330 of three, 40,101: 249 and 230, 77,693: 309 and 411)
+    if (mode == 0 && width == 1 && f > kPairFiles)
+        return all / 4.7 * full + 30.0 < all / 5.6 + chosen / 2.3 + 10.0;
     const double wave = 1.0 + 0.4 * (full - 1.0);
-    const double all = (double)f * r * (double)d * 4e-6, chosen = all / r;      // MB: us at 1 TB/s
-    const double once = (many ? all + chosen : all) / 6.3 * wave + 30.0;
-    const double apart = all / 7.1 + (many ? chosen / 2.7 : chosen / (mode == 1 ? 5.6 : 4.4) * wave) + 10.0;
-    return once < apart;
+    return all / 6.3 * wave + 30.0 < all / 7.1 + chosen / (mode == 1 ? 5.6 : 4.4) * wave + 10.0;
 }
 
 cudaError_t launch_decide(uint32_t *file_neq, const uint8_t *fw, int64_t f, int r, int K, uint32_t *adj,
@@ -394,7 +410,7 @@ cudaError_t launch_round_fused(bool &done, const float *copies, int64_t f, int r
                                int8_t *sel, int mode, float *out, cudaStream_t stream)
 {
     done = false;
-    if (r > 5 || !one_pass_pays(f, r, d, mode, (uintptr_t)copies % 8 == 0 && ld % 2 == 0)) return cudaSuccess;
+    if (r > 5 || !one_pass_pays(f, r, d, mode, load_width(copies, ld))) return cudaSuccess;
     const SweepArgs A{copies, d, ld, (int)f, sel, det, out, file_neq, r, nullptr, nullptr, nullptr, 0};
     switch (r) {
     case 2: return fused<2>(done, A, fw, K, adj, sel, mode, stream);

@@ -30,6 +30,7 @@ namespace aspis {
 constexpr int64_t kPairFiles = 516;         // most files whose tag bytes let two blocks share an SM
 constexpr int64_t kLongFiles = 1200;        // most files whose tag bytes leave a block alone room for long lists
 constexpr int64_t kTagFiles = 1330;         // most files whose tag bytes leave a tile room in a block
+constexpr int64_t kNarrowFiles = 2700;      // most files whose tag bytes fit 64-coordinate tiles (aggregate.cu)
 constexpr int kFewFiles = 36;               // most files whose values one thread sorts in registers (few.cu)
 constexpr int kUnclean = 16;                // in a guessed sel: copies of the file differ
 // Bits of a coordinate that the sweep leaves to fixup_kernel.  They may also

@@ -3,6 +3,8 @@ copies on, by the tiles that the length makes): every step's output against the 
 selections that the sampled coordinates show, for distortions that they miss
 (the aggregate is then made again), for ragged and unaligned rows, and for
 values that need the median's exact passes."""
+import statistics
+
 import numpy as np
 import pytest
 
@@ -202,3 +204,39 @@ def test_few_files_with_many_values():
     for i, s in zip(*np.nonzero(mask)):
         host[i, s, d // 2 + 7 * i] += 5.0
     check(oa, host, d)
+
+
+@pytest.mark.parametrize("K,r,d,extra", [(14, 5, 159_840, 0), (16, 5, 18_312, 2), (31, 3, 77_864, 2), (21, 4, 66_832, 0),
+                                         (24, 3, 32_936, 1), (13, 5, 48_172, 1)])
+def test_round_takes_no_longer_than_its_four_calls(K, r, d, extra):
+    """Where one pass over the copies loses, the round is taken apart: these took
+    7 to 36% longer than check, detect, select and aggregate one after the other
+    when the rule did not know the rows' alignment and how full the waves are."""
+    a = ap.aspis_assign(K, r)
+    d += extra
+    gen = torch.Generator(DEV).manual_seed(2)
+    copies = torch.randn((a.f, 1, d), device=DEV, generator=gen).expand(a.f, r, d).contiguous()
+    buf = ap.RoundBuffers(a, d, DEV)
+
+    def one_call():
+        ap.aspis_round(copies, d, a, buf.file_neq, buf.adj, buf.det, buf.sel, buf.out)
+
+    def four_calls():
+        ap.aspis_check(copies, d, a, buf.file_neq, buf.adj)
+        ap.aspis_detect(buf.adj, K, buf.det)
+        ap.aspis_select(buf.file_neq, buf.det, a, buf.sel)
+        ap.aspis_aggregate(copies, d, a, buf.sel, buf.det, buf.out)
+
+    def timed(call):
+        times = []
+        for _ in range(11):
+            t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            t0.record()
+            call()
+            t1.record()
+            torch.cuda.synchronize()
+            times.append(t0.elapsed_time(t1))
+        return statistics.median(times[2:])
+
+    apart, whole = timed(four_calls), timed(one_call)
+    assert whole < 1.06 * apart, (whole, apart)
