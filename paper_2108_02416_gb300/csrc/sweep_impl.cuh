@@ -299,18 +299,38 @@ sweep_kernel(const SweepArgs A)
             __syncthreads();
             start = cleanest_start(list, f, &start_s);
         }
-        int mine = 0;
-        for (int i = tid; i < f; i += kNT) {
-            const int s = A.sel[i];
-            meta[(i < start ? f : 0) + i - start] =
-                (AVG ? (uint32_t)A.slot_mask[i] : (uint32_t)(s < 0 ? kDropped : s & (kUnclean - 1))) |
-                ((uint32_t)i << 16);
-            mine += AVG ? A.slot_mask[i] != 0 : s >= 0;
+        if constexpr (MODE == MEAN) {
+            // the kept files first, in file order, and the others from the end: a
+            // warp sums the same values in the same order as the separate mean
+            for (int b0 = 0; b0 < f; b0 += kNT) {
+                const int i = b0 + tid, s = i < f ? (int)A.sel[i] : -1;
+                const unsigned m = __ballot_sync(full, s >= 0);
+                if (lane == 0) warp_tot[w] = __popc(m);
+                __syncthreads();
+                int off = n + __popc(m & ((1u << lane) - 1u));
+                for (int q = 0; q < kWarps; ++q) {
+                    off += q < w ? warp_tot[q] : 0;
+                    n += warp_tot[q];
+                }
+                if (i < f)
+                    meta[s >= 0 ? off : f - 1 - (i - off)] =
+                        (uint32_t)(s < 0 ? kDropped : s & (kUnclean - 1)) | ((uint32_t)i << 16);
+                __syncthreads();
+            }
+        } else {
+            int mine = 0;
+            for (int i = tid; i < f; i += kNT) {
+                const int s = A.sel[i];
+                meta[(i < start ? f : 0) + i - start] =
+                    (AVG ? (uint32_t)A.slot_mask[i] : (uint32_t)(s < 0 ? kDropped : s & (kUnclean - 1))) |
+                    ((uint32_t)i << 16);
+                mine += AVG ? A.slot_mask[i] != 0 : s >= 0;
+            }
+            mine = __reduce_add_sync(full, mine);
+            if (lane == 0 && mine) atomicAdd(&n_s, mine);
+            __syncthreads();
+            n = n_s;
         }
-        mine = __reduce_add_sync(full, mine);
-        if (lane == 0 && mine) atomicAdd(&n_s, mine);
-        __syncthreads();
-        n = n_s;
     }
     const uint32_t krank = (uint32_t)((n - 1) / 2);
     // With more files the bins span more than the sample's range, so that the
