@@ -986,12 +986,8 @@ cudaError_t try_launch(bool &launched, const float *copies, int64_t f, int r, in
     const Layout L = make_layout<V, NT, MODE>(f);
     if (L.total > smem_cap()) return cudaSuccess;
     auto kern = aggregate_kernel<V, MINB, W32, MODE, NT, LEAVE>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)L.total);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, L.total);
-    if (e != cudaSuccess) return e;
+    static Residency resident;
+    const int per_sm = resident.blocks(kern, NT, L.total);
     if (per_sm < MINB) return cudaSuccess;        // the next configuration is tried
     const int64_t ntiles = (d + Geo<V>::TC - 1) / Geo<V>::TC;
     int64_t grid = (int64_t)sm_count() * per_sm;
@@ -1006,12 +1002,8 @@ cudaError_t launch_radix(const float *copies, int64_t f, int r, int64_t d, int64
 {
     const size_t smem = (size_t)(256 * 32 + 64) * 4 + ((size_t)f * 2 + 15) / 16 * 16;
     if (smem > smem_cap()) return cudaErrorInvalidValue;
-    cudaError_t e = cudaFuncSetAttribute(median_radix_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, median_radix_kernel, kRadixThreads, smem);
-    if (e != cudaSuccess) return e;
+    static Residency resident;
+    const int per_sm = resident.blocks(median_radix_kernel, kRadixThreads, smem);
     const int64_t ntiles = (d + 31) / 32;
     int64_t grid = (int64_t)sm_count() * (per_sm > 0 ? per_sm : 1);
     if (grid > ntiles) grid = ntiles;
