@@ -206,9 +206,9 @@ file_mean_kernel(const float *__restrict__ copies, int64_t f, int64_t d, int64_t
         const int64_t c0 = (item - i * nchunks) * per;
         const float *rw = copies + i * R * ld;
         float *out = means + i * ldm;
+        if constexpr (VEC) {
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            if constexpr (VEC) {
+            for (int u = 0; u < kU; ++u) {
                 const int64_t c = c0 + ((int64_t)u * kThreads + threadIdx.x) * 4;
                 if (c + 3 < d) {
                     float4 x4[R];
@@ -240,14 +240,21 @@ file_mean_kernel(const float *__restrict__ copies, int64_t f, int64_t d, int64_t
                         out[c + e] = mean_masked<R>(a, m, s0, k);
                     }
                 }
-            } else {
-                const int64_t c = c0 + (int64_t)u * kThreads + threadIdx.x;
-                if (c < d) {
-                    float a[R];
+            }
+        } else {
+            // all loads before the averages, whose branches would part them (455 files
+            // of three, d = 131,073, the whole round: 408 us, 433 one by one)
+            float a[kU][R];
 #pragma unroll
-                    for (int s = 0; s < R; ++s) a[s] = (m >> s) & 1u ? __ldcs(rw + s * ld + c) : 0.f;
-                    out[c] = mean_masked<R>(a, m, s0, k);
-                }
+            for (int u = 0; u < kU; ++u) {
+                const int64_t c = c0 + (int64_t)u * kThreads + threadIdx.x;
+#pragma unroll
+                for (int s = 0; s < R; ++s) a[u][s] = c < d && ((m >> s) & 1u) ? __ldcs(rw + s * ld + c) : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int64_t c = c0 + (int64_t)u * kThreads + threadIdx.x;
+                if (c < d) out[c] = mean_masked<R>(a[u], m, s0, k);
             }
         }
     }
