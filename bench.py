@@ -373,12 +373,17 @@ def captured_kernels(torch, stream, call):
     return kernels
 
 
+# Kernels of a round in one pass: sample, decide, sweep, decide, repair (and the
+# open coordinates of a median); taken apart, at most compare, decide, aggregate
+# and the open coordinates.
+ONE_PASS_KERNELS = 5
+
+
 def round_entry(w, n_sel, kernels, ms, peak, peak_kind, traffic=None):
     """Roofline of the whole round: in one pass every copy is read once and d
     coordinates are written; else the chosen copies are read again."""
     cmp_bytes, agg_bytes = algorithmic_bytes(w, n_sel)
-    one_pass = kernels >= 6        # sample, decide, sweep, decide, repair, (open coordinates)
-    if not one_pass:
+    if kernels < ONE_PASS_KERNELS:
         return hbm_entry("aspis_round (compare, decide, aggregate)", cmp_bytes + agg_bytes, ms,
                          peak, peak_kind)
     return hbm_entry(f"aspis_round in one pass (sweep_kernel<{w.r}>)", cmp_bytes + w.d * 4, ms,

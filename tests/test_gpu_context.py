@@ -1,4 +1,8 @@
-"""What the library remembers of its kernels holds for other threads."""
+"""What the library remembers of its kernels holds for other threads and after the
+device was reset."""
+import os
+import subprocess
+import sys
 import threading
 
 import pytest
@@ -10,6 +14,13 @@ if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 ap = pytest.importorskip("paper_2108_02416_gb300")
 DEV = torch.device("cuda:0")
+
+
+def test_aggregation_after_a_device_reset():
+    here = os.path.dirname(os.path.abspath(__file__))
+    p = subprocess.run([sys.executable, os.path.join(here, "_reset_worker.py")], capture_output=True, text=True,
+                       timeout=300)
+    assert p.returncode == 0 and p.stdout.strip() == "done", p.stdout + p.stderr
 
 
 # one kernel each, with different amounts of shared memory

@@ -1,6 +1,6 @@
 """Full-size parity: the five benchmark workloads at their real sizes, run
-through the C ABI exactly as bench.py runs them (aspis_check, aspis_detect,
-aspis_select, aspis_aggregate on one side stream).
+through the C ABI exactly as bench.py runs them (aspis_round on a side stream, and
+the separate calls after it).
 
 The oracle recomputes every file's agreement word on the host (files are
 streamed through a pinned buffer), then the graph, the maximum cliques and
@@ -64,12 +64,17 @@ def test_fullsize_round(name):
     buf = ap.RoundBuffers(a, w.d, DEV)
     stream = torch.cuda.Stream(device=DEV)
     stream.wait_stream(torch.cuda.current_stream())      # inputs were made on the default stream
+    steps = ap.RoundBuffers(a, w.d, DEV)
     with torch.cuda.stream(stream):
-        ap.aspis_check(copies, w.d, a, buf.file_neq, buf.adj, stream)
-        ap.aspis_detect(buf.adj, w.K, buf.det, stream)
-        ap.aspis_select(buf.file_neq, buf.det, a, buf.sel, stream)
-        ap.aspis_aggregate(copies, w.d, a, buf.sel, buf.det, buf.out, ap.MEDIAN, stream)
+        ap.aspis_round(copies, w.d, a, buf.file_neq, buf.adj, buf.det, buf.sel, buf.out, ap.MEDIAN, stream)
+        ap.aspis_check(copies, w.d, a, steps.file_neq, steps.adj, stream)
+        ap.aspis_detect(steps.adj, w.K, steps.det, stream)
+        ap.aspis_select(steps.file_neq, steps.det, a, steps.sel, stream)
+        ap.aspis_aggregate(copies, w.d, a, steps.sel, steps.det, steps.out, ap.MEDIAN, stream)
     torch.cuda.synchronize()
+    for one, four in ((buf.file_neq, steps.file_neq), (buf.adj, steps.adj), (buf.sel, steps.sel),
+                      (buf.out.view(torch.int32), steps.out.view(torch.int32)), (buf.det[:24], steps.det[:24])):
+        assert torch.equal(one, four)
     det = buf.detection()
     assert det.status == ap.OK
 

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import oracle
-from _gpu_round import as_u32
+from _gpu_round import as_u32, spoil
 
 pytestmark = pytest.mark.gpu
 
@@ -18,28 +18,8 @@ ap = pytest.importorskip("paper_2108_02416_gb300")
 DEV = torch.device("cuda:0")
 
 
-def spoil(u, rng):
-    """Columns of u (uint32 [f, d]) that no tile settles: groups of 32 with 1, 2, 5,
-    6, 7, 12, 17 and 32 of them, of every kind, and single ones at both ends."""
-    f, d = u.shape
-    i = np.arange(f)
-    kinds = [np.zeros(f), np.full(f, 0x3F800000),
-             np.where(i % 2, 0x3F800000, 0xBF800000), np.where(i % 3, 0, 0x80000000),
-             np.where(i % 5, 0, rng.integers(0, 1 << 32, f)), i % 7,
-             np.where(i == f // 2, 0x7FC00001, u[:, 0]), np.where(i % 2, 0x7F800000, 0xFF800000),
-             np.where(i % 2, 0xFFFFFFFF, 0x7FFFFFFF), rng.integers(0, 1 << 32, f),
-             np.where(i % 4, 0xFFFFFFFF, u[:, 0]), np.where(i % 4, 0x7F7FFFFF, 0xFF7FFFFF)]
-    spots = {0, d - 1}
-    for g, many in enumerate([1, 2, 5, 6, 7, 12, 17, 32]):
-        if 32 * g + 32 <= d:
-            spots.update(32 * g + rng.permutation(32)[:many])
-    spots.update(rng.integers(0, d, d // 300))
-    for k, c in enumerate(sorted(spots)):
-        u[:, c] = kinds[(k * 5 + k // len(kinds)) % len(kinds)]
-
-
-# the files' number and the rows' alignment decide which tiles take them and how many
-# that is done by the tile's own block (one tile per SM) or by the kernel after it
+# the files' number, the rows' alignment and d decide which tiles leave them open, and
+# who settles them: the tile's own block (one tile per SM) or the kernel after it
 @pytest.mark.parametrize("K,r", [(8, 3), (15, 3), (12, 4), (16, 3), (18, 3), (12, 6), (20, 3), (21, 3)])
 @pytest.mark.parametrize("d,odd", [(300, 0), (19_600, 0), (19_600, 2), (19_601, 1)])
 def test_open_coordinates(K, r, d, odd):
