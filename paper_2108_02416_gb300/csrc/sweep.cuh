@@ -28,6 +28,7 @@
 namespace aspis {
 
 constexpr int64_t kPairFiles = 516;         // most files whose tag bytes let two blocks share an SM
+constexpr int64_t kSettleFiles = 256;       // most files whose few tiles settle their open coordinates themselves
 constexpr int64_t kLongFiles = 1200;        // most files whose tag bytes leave a block alone room for long lists
 constexpr int64_t kTagFiles = 1330;         // most files whose tag bytes leave a tile room in a block
 constexpr int64_t kNarrowFiles = 2700;      // most files whose tag bytes fit 64-coordinate tiles (aggregate.cu)

@@ -180,9 +180,11 @@ __device__ __forceinline__ int warp_ranked(uint32_t a, uint32_t b, uint32_t cnt,
 }
 
 // The coordinates that a block left open (kOpen in its part of out), at the end
-// of its sweep, where there are so few tiles that fixup_kernel's launch would
-// cost more.  In larger calls the mere presence of this call costs the sweep 5
-// to 9%.  stage: room for 32 coordinates' keys.
+// of its sweep: for few tiles of few files (kSettleFiles), where fixup_kernel's
+// launch costs more (the round of 84 files of three at d = 4,096: 28 us, 31 with
+// fixup_kernel; equal at 220 files, but 36 and 36 at 455 and 55 and 51 at 1,140).
+// In larger calls the mere presence of this call costs the sweep 5 to 9%.  stage:
+// room for 32 coordinates' keys.
 __device__ __noinline__ void settle_open(const SweepArgs &A, uint32_t *stage, const uint32_t *meta, int n,
                                          int64_t t0, int64_t tstep)
 {
@@ -890,9 +892,8 @@ cudaError_t sweep_for(bool &ok, bool &open, const SweepArgs &A, int mode, bool c
     const bool alone = (A.d + TC - 1) / TC <= sm_count();
     cudaError_t e = cudaSuccess;
     if constexpr (R == 1) {
-        if (alone && A.f <= kTagFiles) {
-            e = A.f <= kLongFiles ? try_sweep<R, W, TAGGED, 1, false, 64, true>(ok, A, chained, stream)
-                                  : try_sweep<R, W, TAGGED, 1, false, 32, true>(ok, A, chained, stream);
+        if (alone && A.f <= kSettleFiles) {
+            e = try_sweep<R, W, TAGGED, 1, false, 32, true>(ok, A, chained, stream);
             if (ok) open = false;
             return e;
         }
