@@ -31,9 +31,10 @@
  *   - Gradient copies are one fp32 buffer laid out [f][r][ld]: row (i, s) is
  *     the vector returned by the worker in slot s of file i (slots are in
  *     ascending worker order); only the first d of the ld floats of a row are
- *     read.  ld >= d.  The 128-bit load path is used when the buffer is
- *     16-byte aligned and ld % 4 == 0; otherwise a 4-byte path is used (not
- *     an error).
+ *     used.  ld >= d.  Loads are 128 bits wide when the buffer is 16-byte
+ *     aligned and ld % 4 == 0 (they may touch a row's padding); otherwise the
+ *     compare uses 4-byte loads, the aggregation 8-byte ones when the buffer is
+ *     8-byte aligned and ld is even, else 4-byte ones (not an error).
  *   - Equality of copies is bitwise equality of their fp32 words (+0 != -0;
  *     NaNs equal iff their bit patterns are).
  *   - Workers are 0-based.  Bit k of a worker mask is worker k.  K <= 31.
@@ -195,7 +196,10 @@ aspis_status aspis_aggregate(const float *copies, int64_t d, int64_t ld,
                              aspis_detection *det, int mode, float *out,
                              void *stream);
 
-/* Steps 1-5 back to back on one stream (the whole PS step of one round). */
+/* Steps 1-5 on one stream (the whole PS step of one round): the results are
+ * those of the four calls.  Long rounds guess the selection from a few
+ * coordinates of every copy and compare and aggregate in one pass over the
+ * copies; a distortion outside those coordinates costs a second aggregation. */
 aspis_status aspis_round(const float *copies, int64_t d, int64_t ld,
                          const aspis_assignment *a, uint32_t *file_neq,
                          uint32_t *adj, aspis_detection *det, int8_t *sel,
@@ -249,9 +253,11 @@ aspis_status aspis_round_static(const float *copies, int64_t d, int64_t ld,
  * copy kernel whose SM loads stream over the host link, in eight file-aligned
  * chunks, and each chunk is compared on a library-owned stream (created on
  * first use) as soon as it has landed; other copies of 64 MiB or more are
- * split over four library-owned streams that the stream waits for.  The host
- * buffers must stay valid until the stream is synchronized.  Device
- * buffers are the caller's, as for aspis_round. */
+ * split over four library-owned streams that the stream waits for.  (These
+ * streams end with a cudaDeviceReset of their device, after which this call
+ * must not be made on it again in the same process.)  The host buffers must
+ * stay valid until the stream is synchronized.  Device buffers are the
+ * caller's, as for aspis_round. */
 aspis_status aspis_round_host(const float *host_copies, float *dev_copies,
                               int64_t d, int64_t ld, const aspis_assignment *a,
                               uint32_t *file_neq, uint32_t *adj,

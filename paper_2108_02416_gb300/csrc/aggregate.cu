@@ -1,10 +1,12 @@
-// Step 5 of the PS round for more files than the tiles of sweep_impl.cuh hold
-// tags for (kTagFiles): the coordinate-wise lower median of the chosen copies
-// in narrower tiles or in two passes.
+// Step 5 of the PS round where the 128-coordinate tiles of sweep_impl.cuh are not
+// the better ones (launch_aggregate in round.cu): the coordinate-wise lower median
+// of the chosen copies for more files than those tiles hold tags for (kTagFiles),
+// in narrower tiles or in two passes, and for 517 to 1,330 files in narrower
+// tiles; the mean in narrow tiles.
 //
 // Data path.  A tile is TC = 32*V consecutive coordinates (V = 4, 2 or 1) of
 // all n kept rows.  Lane l of every warp holds coordinates [l*V, l*V + V) of
-// the tile and the 8 warps split the rows: warp w reads rows w, w + 8, ...
+// the tile and the 12 warps split the rows: warp w reads rows w, w + 12, ...
 // straight from global memory with one V-wide load per row, so a warp-wide
 // load is one contiguous 128*V-byte segment of a row.  (Gathering 128-byte
 // segments of 455 rows that lie 45 MB apart runs at about 4.9 TB/s on GB300,
@@ -13,27 +15,27 @@
 // come in batches of kU (8, or 24 for V <= 2 with one CTA per SM) per thread, every
 // register refilled with the next batch's row as soon as it is read, and the
 // last batch of a tile refills with the first rows of the CTA's next tile,
-// whose loads then overlap this tile's remaining phases.  Shared memory holds one tag byte per value, the
-// histograms, the member lists and small per-coordinate state; two CTAs of
-// 12 warps share an SM.
+// whose loads then overlap this tile's remaining phases.  Shared memory holds one
+// tag byte per value (not in two passes), the histograms, the member lists and
+// small per-coordinate state; two CTAs share an SM where it suffices.
 //
 // Lower median, exact (IEEE totalOrder through a monotone uint32 key; the key
 // map is a bijection, so the output has the chosen element's bits).  Per
 // tile:
 //   S   sample: key range of the first two rows of every warp (24 values per
 //       coordinate).
-//   VH  value-space histogram of every value: bins 1..125 evenly over the
-//       sample range, 0 and 126 catch everything below / above (vbin_bits);
+//   VH  value-space histogram of every value: bins 1..253 evenly over the
+//       sample range, 0 and 254 catch everything below / above (vbin_bits);
 //       each value's bin is kept as a tag byte; NaNs are detected.  Counters
-//       are the 16-bit halves of words in per-lane columns, so the 32 shared
-//       atomics of a warp instruction hit 32 different banks.
+//       are the 16-bit halves (V = 4: the bytes) of words in per-lane columns,
+//       so the 32 shared atomics of a warp instruction hit 32 different banks.
 //   B   bin search: per-warp partial sums over kBPW bins, then one thread per
 //       coordinate finds the bin that holds the target rank, the rank inside
 //       it and its count.
 //   VC  right after the bin search, four tag bytes are compared per word; the
 //       bin's members (about n/80) are copied from global memory (the tile is
-//       still in L2) into a list of at most CAP values per coordinate (4096 / TC) by
-//       4-byte cp.async; they land during the next tile's sweep, after which
+//       still in L2) into a list of at most CAP values per coordinate by 4-byte
+//       cp.async (two passes: taken from the second one's registers); they land during the next tile's sweep, after which
 //       one thread per coordinate sorts its keys in registers.
 // Exact fallback for the coordinates that need it (NaN seen, degenerate or
 // non-finite sample range, more than CAP members in the bin), values
@@ -129,6 +131,7 @@ __global__ void __launch_bounds__(NT, MINB)
 aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, int64_t ld,
                  const int8_t *__restrict__ sel, aspis_detection *det, float *__restrict__ out)
 {
+    static_assert(V < 4 || MODE != 0, "the tags of 128-coordinate tiles are sweep_impl.cuh's");
     using G = Geo<V>;
     using T = typename Vec<V>::T;
     constexpr int TC = G::TC, NP = G::NP, SHB = G::SHB, RPW = G::RPW;
@@ -461,8 +464,6 @@ aggregate_kernel(const float *__restrict__ copies, int64_t f, int r, int64_t d, 
                 if constexpr (V == 4) {
                     nan_check(nanf, __uint_as_float(x.x), __uint_as_float(x.y),
                               __uint_as_float(x.z), __uint_as_float(x.w));
-                    if constexpr (MODE == 0)
-                        tags[(j * kWarps + w) * 32 + lane] = pack4(bb[0], bb[1], bb[2], bb[3]);
                 } else if constexpr (V == 2) {
                     nan_check(nanf, __uint_as_float(x.x), __uint_as_float(x.y),
                               __uint_as_float(x.x), __uint_as_float(x.y));

@@ -1,4 +1,4 @@
-// Pieces of the coordinate-wise aggregation (aggregate.cu): the totalOrder
+// Pieces of the coordinate-wise aggregation: the totalOrder
 // key map, the value-space bin map, tag matching, compensated sums and the
 // search modes of the lower median.
 #pragma once
@@ -31,7 +31,7 @@ __device__ __forceinline__ uint32_t from_key(uint32_t k)
 // [0, 1] (fma with saturation: NaN gives +0), then 2^23 + rint(254*y), whose
 // low byte is the bin 0..254.  Both steps are correctly rounded and
 // non-decreasing, so the map is monotone in the IEEE totalOrder of every
-// non-NaN x (+0 and -0 share a bin) and always lands in 0..126, whatever s
+// non-NaN x (+0 and -0 share a bin) and always lands in 0..254, whatever s
 // and c are.  NaNs are detected separately.
 __device__ __forceinline__ uint32_t vbin_bits(float x, float s, float c)
 {

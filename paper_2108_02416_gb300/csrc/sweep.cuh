@@ -18,7 +18,7 @@
 // More than kTagFiles files leave no room for tags: the sweep then only counts,
 // and a second pass over the chosen rows lists the members.  (Sharing a tile
 // among the blocks of a cluster, counters and members exchanged through
-// distributed shared memory, kept one pass but cost 15 to 25 us per tile: 6.9
+// distributed shared memory, kept one pass but cost 15 to 25 us per tile: 7.0
 // against 6.2 ms at 3,003 files of five copies and d = 2^19.)
 #pragma once
 

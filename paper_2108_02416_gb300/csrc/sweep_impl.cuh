@@ -134,8 +134,8 @@ __device__ __forceinline__ uint32_t vdiff(const uint4 &a, const uint4 &b)
 // distortions, so some window has few even where a quarter of all files is
 // distorted.  (A sample spread over the file order is as good, but rows taken
 // from all over the copies at a tile's start cost 7 to 10% of the pass at 61
-// GB, read once or twice, prefetched or not.)  Called by the whole block; n <=
-// kTileFiles.
+// GB, read once or twice, prefetched or not.)  Called by the whole block; marked
+// holds n words, in the list, which every layout makes long enough.
 __device__ __forceinline__ int cleanest_start(const uint32_t *marked, int n, int *best)
 {
     if (n < 2 * kSample) return 0;
@@ -898,17 +898,21 @@ cudaError_t sweep_for(bool &ok, bool &open, const SweepArgs &A, int mode, bool c
             return e;
         }
     }
-    if (A.f <= kTagFiles) {
-        if (!alone && A.f <= kPairFiles) {
-            e = try_sweep<R, W, TAGGED, 2>(ok, A, chained, stream);
-            if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 2, false, 16>(ok, A, chained, stream);
-        }
-        if (e == cudaSuccess && !ok)
+    if ((!alone || R == 2) && A.f <= kPairFiles) {
+        e = try_sweep<R, W, TAGGED, 2>(ok, A, chained, stream);
+        if (e == cudaSuccess && !ok) e = try_sweep<R, W, TAGGED, 2, false, 16>(ok, A, chained, stream);
+    }
+    if constexpr (R == 2) {
+        return e;                     // two copies: at most 465 files
+    } else {
+        if (e != cudaSuccess || ok) return e;
+        if (A.f <= kTagFiles) {
             e = A.f <= kLongFiles ? try_sweep<R, W, TAGGED, 1, false, 64>(ok, A, chained, stream)
                                   : try_sweep<R, W, TAGGED, 1>(ok, A, chained, stream);
-        if (e != cudaSuccess || ok) return e;
+            if (e != cudaSuccess || ok) return e;
+        }
+        return try_sweep<R, W, TWO_PASS, 2>(ok, A, chained, stream);
     }
-    return try_sweep<R, W, TWO_PASS, 2>(ok, A, chained, stream);
 }
 
 }  // namespace
@@ -930,9 +934,9 @@ cudaError_t launch_sweep_averages(bool &ok, const SweepArgs &A, cudaStream_t str
     const bool chained = false;
     cudaError_t e = cudaSuccess;
     if ((A.d + TC - 1) / TC > sm_count()) e = try_sweep<R, 4, TAGGED, 2, true>(ok, A, chained, stream);
-    if (e == cudaSuccess && !ok)
-        e = A.f <= kLongFiles ? try_sweep<R, 4, TAGGED, 1, true, 64>(ok, A, chained, stream)
-                              : try_sweep<R, 4, TAGGED, 1, true>(ok, A, chained, stream);
+    if (e != cudaSuccess || ok) return e;
+    if (R == 2 || A.f <= kLongFiles) return try_sweep<R, 4, TAGGED, 1, true, 64>(ok, A, chained, stream);
+    if constexpr (R > 2) e = try_sweep<R, 4, TAGGED, 1, true>(ok, A, chained, stream);
     return e;
 }
 
