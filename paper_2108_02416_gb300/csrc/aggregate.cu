@@ -35,8 +35,9 @@
 //   VC  right after the bin search, four tag bytes are compared per word; the
 //       bin's members (about n/80) are copied from global memory (the tile is
 //       still in L2) into a list of at most CAP values per coordinate by 4-byte
-//       cp.async (two passes: taken from the second one's registers); they land during the next tile's sweep, after which
-//       one thread per coordinate sorts its keys in registers.
+//       cp.async (two passes: taken from the second one's registers); they
+//       land during the next tile's sweep, after which one thread per
+//       coordinate sorts its keys in registers.
 // Exact fallback for the coordinates that need it (NaN seen, degenerate or
 // non-finite sample range, more than CAP members in the bin), values
 // re-read from global memory:

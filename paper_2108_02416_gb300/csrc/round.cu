@@ -24,8 +24,8 @@
 // det->success (bit 1), taken back by the repair's last block, open
 // coordinates as a bit pattern in out.
 //
-// The sweep is bound by HBM (61.0 GB in 9.5 ms = 6.4 TB/s at 455 files of
-// three copies and 11.2M coordinates; the separate passes took 8.7 + 4.9 ms).
+// The sweep is bound by HBM (61.0 GB in 9.8 ms = 6.2 TB/s at 455 files of
+// three copies and 11.2M coordinates; the separate passes take 8.7 + 4.4 ms).
 // With one copy per file (R = 1) it is the separate aggregation: 0.43 ms at
 // 455 files and 2^20 coordinates.
 #include "aspis_internal.cuh"

@@ -31,11 +31,11 @@ enum Mode { TAGGED = 0, MEAN = 1, TWO_PASS = 2 };
 // List entries per coordinate (CAP; the two-pass median's bins are wider).  A
 // bin has n / 120 members on average.  Two blocks share the SM up to 456 files
 // with 32 entries and up to kPairFiles with 16, which are hardly ever exceeded
-// there by continuous values; values kept in 16 bits, whose grid is coarser than
-// the bins, do exceed them (495 files, d = 524,288: 251 us, 647 with gradients of
-// bf16; with a block alone 390 and 440).  A block alone takes 64 where they fit
-// (kLongFiles): of such values at 816 files it leaves 881 coordinates of 524,288
-// open, not 56,173 (672 us, not 1,136).
+// there by continuous values (495 files, d = 1,048,576: 456 us, 723 with a block
+// alone); values kept in 16 bits, whose grid is coarser than the bins, do exceed
+// them (1,211 and 820).  A block alone takes 64 where they fit (kLongFiles): of
+// such values at 816 files it leaves 881 coordinates of 524,288 open, not 56,173
+// (672 us, not 1,136).
 template <int MODE, int CAP>
 __host__ __device__ constexpr int list_cap() { return MODE == TWO_PASS ? 96 : CAP; }
 constexpr int kHistWords = kVB * 32;        // four 8-bit counters per (bin, lane)
